@@ -164,6 +164,14 @@ dabnn_status fill_args(BConvArgs& g, const uint64_t* a, dabnn_shape in, const ui
   return DABNN_OK;
 }
 
+// Packed-weight calls that run on the tensor-core engine (same integers, see tc_bits_worthwhile), unless a measurement
+// run has fixed the loop or the tile, or the call belongs to a chained forward whose caller gave no expanded weights.
+bool tensor_route(dabnn_shape in, const uint64_t* w, int O, dabnn_conv cv, int epi) {
+  if (!aligned(w, 16)) return false;  // (its weight rows are fetched with bulk copies)
+  if (g_conv_variant != 0 || g_conv_tile != 0 || g_chain_launch) return false;
+  return tc_bits_worthwhile(in, O, cv, epi);
+}
+
 }  // namespace
 
 int sm_count() {
@@ -229,6 +237,10 @@ extern "C" dabnn_status dabnn_bconv2d(const uint64_t* a_packed, dabnn_shape in, 
   if (!out) return DABNN_ERR_NULL;
   if (out_layout != DABNN_NCHW && out_layout != DABNN_NHWC) return DABNN_ERR_SHAPE;
   if (!aligned(out, 4)) return DABNN_ERR_ALIGNMENT;
+  if (tensor_route(in, w_packed, O, cv, EPI_I32)) {
+    s = tc_bits_bconv2d(a_packed, in, w_packed, O, cv, out, out_layout == DABNN_NCHW, as_stream(stream));
+    if (s != DABNN_ERR_UNSUPPORTED) return s;
+  }
   g.out = out;
   g.out_nchw = out_layout == DABNN_NCHW;
   return launch_epi<EPI_I32>(g, as_stream(stream));
@@ -256,6 +268,10 @@ extern "C" dabnn_status dabnn_bconv2d_bn_sign_pack(const uint64_t* a_packed, dab
   if (s != DABNN_OK) return s;
   if (!scale || !shift || !out_packed) return DABNN_ERR_NULL;
   if (!aligned(scale, 4) || !aligned(shift, 4) || !aligned(out_packed, 8)) return DABNN_ERR_ALIGNMENT;
+  if (tensor_route(in, w_packed, O, cv, EPI_BNPACK)) {
+    s = tc_bits_bn_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, out_packed, as_stream(stream));
+    if (s != DABNN_ERR_UNSUPPORTED) return s;
+  }
   g.scale = scale; g.shift = shift;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
   return launch_epi<EPI_BNPACK>(g, as_stream(stream));
@@ -272,6 +288,10 @@ extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed,
   if (!aligned(scale, 4) || !aligned(shift, 4) || !aligned(residual, 4) || !aligned(y_out, 4) ||
       !aligned(out_packed, 8))
     return DABNN_ERR_ALIGNMENT;
+  if (tensor_route(in, w_packed, O, cv, EPI_BIREAL)) {
+    s = tc_bits_bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed, as_stream(stream));
+    if (s != DABNN_ERR_UNSUPPORTED) return s;
+  }
   g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
   return launch_epi<EPI_BIREAL>(g, as_stream(stream));

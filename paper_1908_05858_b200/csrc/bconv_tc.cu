@@ -6,10 +6,10 @@
 // the block-scaled kind::mxf4 with every scale factor set to 1.0 (ue8m0 127).  Products are +-1 and the fp32
 // accumulator adds at most K < 2^24 of them, so the result is the exact integer.  HBM still holds one bit per value.
 //
-//   * Weights: expanded once (dabnn_tc_prepare_weights) to e2m1 rows of 16 bytes = 32 channels, stored in blocks of 32
-//     output channels ([O/32][tap][C/32][32][16 B]); a persistent CTA copies the rows of its output channels into the
-//     UMMA K-major, no-swizzle core-matrix layout in shared memory once and keeps them for all its pixel tiles -- as
-//     many channel tiles as fit, so that a tile of activations is expanded once for all of them.
+//   * Weights: packed words in HBM.  A persistent CTA fetches the packed rows of its output channels with bulk copies,
+//     expands them once to e2m1 rows of 16 bytes = 32 channels in the UMMA K-major, no-swizzle core-matrix layout in shared
+//     memory and keeps them for all its pixel tiles -- as many channel tiles as fit, so that a tile of activations is
+//     expanded once for all of them.
 //   * CTA pairs: where the launch is large enough, two CTAs of a cluster share every MMA (cta_group::2, M = 256: each
 //     CTA's 128 rows against N columns of which each CTA holds half).  Per MMA a CTA then reads half the weights from
 //     its shared memory -- the tensor pipe's operand reads are what saturates shared memory in the one-CTA form -- and
@@ -64,7 +64,10 @@ int g_tc_max_ctas = 0;          // host: CTAs per launch at most (0: one per SM)
 
 struct TcArgs {
   const uint64_t* a;
-  const uint8_t* w_tc;
+  const uint64_t* w;   // packed weights [O][taps][Cw], 16-byte aligned
+  uint64_t w_tail;     // the bits of a pixel's last word that are channels
+  int raw_off;         // where a CTA's packed weight rows wait for their expansion, in bytes from the first activation buffer
+  int raw_first;       // ... and the first fill of an activation buffer (0 or 1) that has to wait for it
   int N, H, W, Cw, C;
   int O, kh, kw, ph, pw, OH, OW;
   int S;               // stride (1 or 2, both axes)
@@ -103,10 +106,6 @@ struct TcArgs {
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -191,6 +190,17 @@ __device__ __forceinline__ uint4 expand32(uint32_t w) {
   return make_uint4(lo.x, lo.y, hi.x, hi.y);
 }
 
+// Expanded nibbles of the channels whose bit in `valid` is 0 become e2m1 0.0: they contribute nothing.  The validity bits go
+// through the same expansion (and so the same channel order): 0xA marks a live nibble.
+__device__ __forceinline__ uint4 mask_channels(uint4 bytes, uint32_t valid) {
+  const uint4 v = expand32(valid);
+  bytes.x &= ((v.x >> 3) & 0x11111111u) * 0xFu;
+  bytes.y &= ((v.y >> 3) & 0x11111111u) * 0xFu;
+  bytes.z &= ((v.z >> 3) & 0x11111111u) * 0xFu;
+  bytes.w &= ((v.w >> 3) & 0x11111111u) * 0xFu;
+  return bytes;
+}
+
 // 256-bit global store / load (32-byte aligned): a lane writes a whole 32-byte sector of its output row at once.
 // The load (the fp32 residual stream, read once) does not allocate in L1: measured 3 % on the whole Bi-Real forward.
 __device__ __forceinline__ void st_global_v8(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f,
@@ -262,6 +272,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   constexpr int B_MMA_DONE = 0, B_TMEM_FREE = 4, B_A_FULL = 8, B_A_FREE = 12, B_W_FULL = 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 160);
   volatile int* s_fail = reinterpret_cast<volatile int*>(misc + 168);
+  constexpr int B_RAW = 19, B_EXPANDED = 22;  // the packed weight rows have landed / have been expanded
   // [32 + 4 * e ..]: `res_full` of epilogue warp e's ring of residual chunks
   constexpr int B_RES_FULL = 32;
   float* s_scale = reinterpret_cast<float*>(misc + TC_SMEM_HDR);  // [nres][NT] this CTA's channels
@@ -278,82 +289,120 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   const long long mt_end = PAIR ? (g.m_tiles + 1) / 2 * 2 : g.m_tiles;
 
   if (g.chained) chain_trigger();  // the successor may start as CTAs of this launch leave (it waits for all of them itself)
-  if (EPI == EPI_BIREAL) {
-    for (int i = tid; i < nres_here * NT; i += TC_THREADS) {
-      const int o = (ng * g.nres + i / NT) * NT + (i % NT);
-      s_scale[i] = (o < g.O) ? g.scale[o] : 0.0f;
-      s_shift[i] = (o < g.O) ? g.shift[o] : 0.0f;
-    }
-  }
-  if (EPI == EPI_BNPACK) {
-    // The sign of fmaf(acc, scale, shift) as a threshold on the integer acc: fmaf is monotone in acc (the exact value is,
-    // and rounding keeps order), so { acc in [-K, K] : fmaf(acc, scale, shift) < 0 } is empty, everything, a prefix
-    // (scale > 0) or a suffix (scale < 0) of the range -- also for infinite or NaN scale / shift, where the comparison is
-    // false wherever the value is NaN.  A bisection with the very fmaf finds the boundary; the epilogue then needs one
-    // compare per value: bit = (acc <= T) xor flip, with T in s_scale and one flip bit per channel in s_shift's place.
-    uint32_t* s_flip = reinterpret_cast<uint32_t*>(s_shift);
-    const int K = g.kh * g.kw * g.C;
-    for (int i = tid; i < nres_here * NT; i += TC_THREADS) {  // (whole warps: NT is a multiple of 32)
-      const int o = (ng * g.nres + i / NT) * NT + (i % NT);
-      const float sc = (o < g.O) ? g.scale[o] : 0.0f, sh = (o < g.O) ? g.shift[o] : 0.0f;
-      auto neg = [&](int a) { return __fmaf_rn((float)a, sc, sh) < 0.0f; };
-      const bool first = neg(-K), last = neg(K);
-      float T;
-      uint32_t flip = 0;
-      if (first == last) {
-        T = first ? (float)(K + 1) : (float)(-K - 1);  // everything / nothing
-      } else {
-        int lo = -K, hi = K;  // neg(lo) == first, neg(hi) == last
-        while (hi - lo > 1) {
-          const int mid = lo + ((hi - lo) >> 1);
-          if (neg(mid) == first) lo = mid;
-          else hi = mid;
-        }
-        T = (float)lo;        // prefix: negative for acc <= lo; suffix: negative for acc >= hi, i.e. not (acc <= lo)
-        flip = first ? 0u : 1u;
+  // Start-up, the roles side by side (a launch of one or two tiles per CTA is mostly this): warp 12 initialises the barriers
+  // and requests the packed weight rows, warp 0 allocates tensor memory, all others derive the per-channel constants.
+  const bool thirds = g.kh == 3 && g.kw == 3;          // a 3x3 filter's weights become ready one row of taps at a time
+  const int rb_n = nres_here * (WR / 8);               // blocks of 8 weight rows of this CTA
+  if (warp == 12) {
+    if (lane == 0) {
+      for (int i = 0; i < TC_MAX_BUFS; i++) {
+        mbar_init(smem_u32(&bars[B_MMA_DONE + i]), 1);
+        mbar_init(smem_u32(&bars[B_TMEM_FREE + i]), (g.epi2 ? 8 : 4) * PEERS);  // one arrival per epilogue warp
+        mbar_init(smem_u32(&bars[B_A_FULL + i]), 4 * PEERS + (uint32_t)g.extra_arrivals);  // one arrival per producer warp
+        mbar_init(smem_u32(&bars[B_A_FREE + i]), 1);
       }
-      s_scale[i] = T;
-      const uint32_t mask = __ballot_sync(0xFFFFFFFFu, flip != 0);
-      if (lane == 0) s_flip[i >> 5] = mask;
+      // one arrival per expanded block of weight rows; the first third also counts the four warps that write scale factors
+      for (int i = 0; i < 3; i++) mbar_init(smem_u32(&bars[B_W_FULL + i]), (uint32_t)(rb_n + (i == 0 ? 4 : 0)) * PEERS);
+      mbar_init(smem_u32(&bars[B_RAW]), 1);
+      mbar_init(smem_u32(&bars[B_EXPANDED]), (uint32_t)(thirds ? 3 * rb_n : rb_n));
+      if (RES_TMA)
+        for (int i = 0; i < 8 * TC_RING_MAX; i++) mbar_init(smem_u32(&bars[B_RES_FULL + i]), 1);  // the warp's issuing lane
+      *s_fail = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      // the packed rows of each resident channel tile: one bulk copy (the tensor starts on 16 bytes and a tile's rows are a
+      // multiple of 32, so every block does; an odd last word, where O cuts a tile, is copied by hand)
+      const int K64 = g.kh * g.kw * g.Cw;
+      const uint32_t bar = smem_u32(&bars[B_RAW]);
+      auto block = [&](int r, const uint64_t*& src, uint8_t*& dst) {  // bytes of resident tile r's rows (0: all beyond O)
+        const int col0 = (ng * g.nres + r) * NT + (int)rank * WR;
+        src = g.w + (long long)col0 * K64;
+        dst = a_s + g.raw_off + (size_t)r * WR * K64 * 8;
+        return (uint32_t)(max(min(WR, g.O - col0), 0) * K64) * 8u;
+      };
+      const uint64_t* src;
+      uint8_t* dst;
+      uint32_t total = 0;
+#pragma unroll 1
+      for (int r = 0; r < nres_here; r++) {
+        const uint32_t bytes = block(r, src, dst);
+        total += bytes & ~15u;
+        if (bytes & 15u) *reinterpret_cast<uint64_t*>(dst + (bytes & ~15u)) = src[bytes / 8 - 1];
+      }
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(total) : "memory");
+#pragma unroll 1
+      for (int r = 0; r < nres_here; r++) {
+        const uint32_t bytes = block(r, src, dst) & ~15u;
+        if (bytes != 0)
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+                       "l"(src), "r"(bytes), "r"(bar)
+                       : "memory");
+      }
+    }
+    __syncwarp();
+  } else {
+    if (warp == 0) {
+      if (PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"((uint32_t)TC_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+      } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"((uint32_t)TC_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+      }
+    }
+    if (EPI == EPI_BIREAL) {
+      for (int i = tid; i < nres_here * NT; i += TC_THREADS - 32) {
+        const int o = (ng * g.nres + i / NT) * NT + (i % NT);
+        s_scale[i] = (o < g.O) ? g.scale[o] : 0.0f;
+        s_shift[i] = (o < g.O) ? g.shift[o] : 0.0f;
+      }
+    }
+    if (EPI == EPI_BNPACK) {
+      // The sign of fmaf(acc, scale, shift) as a threshold on the integer acc: fmaf is monotone in acc (the exact value is,
+      // and rounding keeps order), so { acc in [-K, K] : fmaf(acc, scale, shift) < 0 } is empty, everything, a prefix
+      // (scale > 0) or a suffix (scale < 0) of the range -- also for infinite or NaN scale / shift, where the comparison is
+      // false wherever the value is NaN.  A bisection with the very fmaf finds the boundary; the epilogue then needs one
+      // compare per value: bit = (acc <= T) xor flip, with T in s_scale and one flip bit per channel in s_shift's place.
+      uint32_t* s_flip = reinterpret_cast<uint32_t*>(s_shift);
+      const int K = g.kh * g.kw * g.C;
+      for (int i = tid; i < nres_here * NT; i += TC_THREADS - 32) {  // (whole warps: NT is a multiple of 32)
+        const int o = (ng * g.nres + i / NT) * NT + (i % NT);
+        const float sc = (o < g.O) ? g.scale[o] : 0.0f, sh = (o < g.O) ? g.shift[o] : 0.0f;
+        auto neg = [&](int a) { return __fmaf_rn((float)a, sc, sh) < 0.0f; };
+        const bool first = neg(-K), last = neg(K);
+        float T;
+        uint32_t flip = 0;
+        if (first == last) {
+          T = first ? (float)(K + 1) : (float)(-K - 1);  // everything / nothing
+        } else {
+          int lo = -K, hi = K;  // neg(lo) == first, neg(hi) == last
+          while (hi - lo > 1) {
+            const int mid = lo + ((hi - lo) >> 1);
+            if (neg(mid) == first) lo = mid;
+            else hi = mid;
+          }
+          T = (float)lo;        // prefix: negative for acc <= lo; suffix: negative for acc >= hi, i.e. not (acc <= lo)
+          flip = first ? 0u : 1u;
+        }
+        s_scale[i] = T;
+        const uint32_t mask = __ballot_sync(0xFFFFFFFFu, flip != 0);
+        if (lane == 0) s_flip[i >> 5] = mask;
+      }
     }
   }
-  if (tid == 0) {
-    for (int i = 0; i < TC_MAX_BUFS; i++) {
-      mbar_init(smem_u32(&bars[B_MMA_DONE + i]), 1);
-      mbar_init(smem_u32(&bars[B_TMEM_FREE + i]), (g.epi2 ? 8 : 4) * PEERS);  // one arrival per epilogue warp
-      mbar_init(smem_u32(&bars[B_A_FULL + i]), 4 * PEERS + (uint32_t)g.extra_arrivals);  // one arrival per producer warp
-      mbar_init(smem_u32(&bars[B_A_FREE + i]), 1);
-    }
-    for (int i = 0; i < 3; i++) mbar_init(smem_u32(&bars[B_W_FULL + i]), TC_THREADS * PEERS);
-    if (RES_TMA)
-      for (int i = 0; i < 8 * TC_RING_MAX; i++) mbar_init(smem_u32(&bars[B_RES_FULL + i]), 1);  // the warp's issuing lane
-    *s_fail = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    if (PAIR) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                   "r"((uint32_t)TC_TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                   "r"((uint32_t)TC_TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-  }
-  // The start-up barrier: barriers initialised (in both CTAs of a pair, before either signals the other's) and the
-  // tensor-memory address published.  Each warp passes it once, as late as its role allows: the weight copy and the
-  // producers' first requests for activation bits are already in flight by then.
+  // The start-up barrier: barriers initialised (in both CTAs of a pair, before either signals the other's), per-channel
+  // constants written and the tensor-memory address published.
   auto prologue_sync = [&]() {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     if (PAIR) cluster_sync_all();
     else __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   };
-  const bool is_producer = warp >= 4 && warp < 8;
-  uint32_t tmem_base = 0;
+  prologue_sync();
+  const uint32_t tmem_base = *tmem_slot;
   // barriers that both CTAs of a pair signal live in the leader
   const uint32_t bar_tmem_free0 = PAIR ? leader_addr(smem_u32(&bars[B_TMEM_FREE])) : smem_u32(&bars[B_TMEM_FREE]);
   const uint32_t bar_a_full0 = PAIR ? leader_addr(smem_u32(&bars[B_A_FULL])) : smem_u32(&bars[B_A_FULL]);
@@ -362,63 +411,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     if (PAIR) mbar_arrive_cluster(bar);
     else mbar_arrive(bar);
   };
-  {
-    // Resident weights: rows [rank * WR, +WR) of every channel tile of this group, one (tile, tap, 32-channel group)
-    // block of WR rows per warp and step; the source holds blocks of 32 output channels.  The producers do not wait
-    // for their share until their first tile's rows are out, so the copy overlaps the first expansion.
-    // The copy goes in three groups, thirds of the (tap, 32-channel group) blocks in issue order -- for a 3x3 filter
-    // one row of taps each -- with a barrier per group: the first MMAs start when the first third has landed.
-    const int TG = g.kh * g.kw * (g.C >> 5);
-#pragma unroll 1
-    for (int j = 0; j < 3; j++) {
-      const int lo = TG * j / 3, cnt = TG * (j + 1) / 3 - lo;
-      for (int idx = warp; idx < nres_here * cnt; idx += TC_THREADS / 32) {
-        const int r = idx / cnt, tg = lo + idx - r * cnt;
-        const int col0 = (ng * g.nres + r) * NT + (int)rank * WR;
-        uint8_t* dst = w_s + (size_t)(r * TG + tg) * WR * 16;
-        for (int n = lane; n < WR; n += 32) {
-          const int col = col0 + n;
-          cp_async16(smem_u32(dst + n * 16), g.w_tc + (((size_t)(col >> 5) * TG + tg) * 32 + (col & 31)) * 16);
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-  }
-  // this thread's share of each third has landed -> one arrival on that third's barrier
-  auto weights_arrive = [&]() {
-    asm volatile("cp.async.wait_group 2;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    arrive(bar_w_full);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    arrive(bar_w_full + 8u);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    arrive(bar_w_full + 16u);
-  };
-  // (chained launches: nothing above reads or writes what the previous kernel of the stream produces or still reads; the
-  // activation bits, the residual and every output come after this point.  A no-op in an ordinary launch.)
-  chain_wait();
-  if (!is_producer) {
-    prologue_sync();
-    tmem_base = *tmem_slot;
-  }
-  if (warp < 4 || warp >= 8) {
-    if (warp < 4) {
-      // every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout
-      const uint32_t one = 0x7F7F7F7Fu;
-      for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
-        const uint32_t taddr = tmem_base + ((uint32_t)(32 * warp) << 16) + (uint32_t)c;
-        asm volatile(
-            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
-            "r"(one)
-            : "memory");
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    weights_arrive();  // one arrival per thread of the CTA (pair) in all: weights (by thirds) and scale factors are in place
-  }
+  // (chained launches: nothing above reads or writes what the previous kernel of the stream produces or still reads; a warp
+  // waits for that kernel where it first touches the activation bits, the residual or an output.  A no-op in an ordinary launch.)
 
   if (warp == 12) {
     // ================= MMA issue: one thread (of the leader CTA) ==================================================
@@ -494,7 +488,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
               mma(d_tmem, a_lo + (uint32_t)kb * a_stp, b_base + ((uint32_t)t * tap_blocks + (uint32_t)kb) * b_step, (t | kb) ? 1u : more);
           }
         } else {
-          if (!KG && first && !(wait(smem_u32(&bars[B_W_FULL + 1]), 0) && wait(smem_u32(&bars[B_W_FULL + 2]), 0))) *s_fail = 1;
           uint32_t b_tap = b_base, accumulate = more;
           for (int ti = 0; ti < g.kh; ti++)
             for (int tj = 0; tj < g.kw; tj++, b_tap += tap_blocks * b_step) {
@@ -510,8 +503,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       uint32_t ab = 0, a_phase = 0;  // A buffer of this tile and the parity of its `a_full` phase
       uint32_t accb = 0, acc_phase = 0;  // accumulator of this round and the parity of its uses so far
       int ar = 0;                    // accumulator rounds so far: one per (tile, resident channel tile)
-      bool ok = wait(smem_u32(&bars[B_W_FULL]), 0);  // first third of the resident weights, and the scale factors
-      if (KG) ok = ok && wait(smem_u32(&bars[B_W_FULL + 1]), 0) && wait(smem_u32(&bars[B_W_FULL + 2]), 0);  // ... all of them
+      bool ok = wait(smem_u32(&bars[B_W_FULL]), 0);  // first third of the resident weights (all of a filter that is not 3x3), and the scale factors
+      if (KG && thirds) ok = ok && wait(smem_u32(&bars[B_W_FULL + 1]), 0) && wait(smem_u32(&bars[B_W_FULL + 2]), 0);  // ... all of them
       if (!ok) *s_fail = 1;
       if constexpr (KG) {
 #pragma unroll 1
@@ -658,6 +651,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       }
     };
 
+    {
+      // every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout (each warp: its quarter of the rows)
+      const uint32_t one = 0x7F7F7F7Fu;
+#pragma unroll 1
+      for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
+        const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c;
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+            "r"(one)
+            : "memory");
+      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) arrive(bar_w_full);
+    }
+    chain_wait();
     int it = 0;
     // Per tile: wait until the A buffer is free, expand the rows held in `cur`, hand them over, move the next tile's
     // bits (requested one tile ago, so they have landed) from `nxt` into `cur`, and request the tile after that into
@@ -670,7 +680,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       long long mt = mt_first;
       prefetch(cur, cwc);  // (rows of a tile beyond the last one are beyond the batch: nothing is read for them)
       if (TWO_SETS) prefetch(nxt, cwc);
-      prologue_sync();
       uint32_t ab = 0, use_phase = 0;  // A buffer of this tile and the parity of the number of times it has been filled
       bool stop = false;
 #pragma unroll 1
@@ -679,16 +688,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       for (int grp = 0; grp < (KG ? g.kgroups : 1); grp++, it++) {  // (KG: a tile's channel groups, one A buffer each)
         // its last reader: all MMAs of the tile that used it, signalled through `a_free` (in both CTAs of a pair)
         // (the decision is taken by the warp as a whole, so that its lanes stay together for the warp-wide steps below)
+        // (the packed weight rows are in the buffers from the second -- or the first -- one on until all are expanded)
+        if (it == g.raw_first &&
+            !__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_EXPANDED]), 0, s_fail, g.wait_polls))) { *s_fail = 1; stop = true; break; }
         if (it >= g.abufs && !__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_A_FREE + ab]), use_phase ^ 1u, s_fail, g.wait_polls))) { *s_fail = 1; stop = true; break; }
         expand(cur, a_s + (size_t)ab * a_bytes, cwc);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
         __syncwarp();  // every lane's rows are written and fenced: one arrival stands for the warp
         if (lane == 0) arrive(bar_a_full0 + 8u * (uint32_t)ab);
-        if (it == 0) {
-          // the first tile's rows went out before anything else: a short launch is all start-up.  Now this thread's
-          // share of the weights.
-          weights_arrive();
-        }
         if (TWO_SETS) {
 #pragma unroll
           for (int h = 0; h < SPT; h++) {
@@ -707,10 +714,57 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     else if (g.Cw == 1) run(IntC<1>{});
     else if (g.Cw == 2) run(IntC<2>{});
     else if (g.Cw <= 4) run(IntC<4>{});
-    else if constexpr (PCW > 4) run(IntC<8>{});
-    else prologue_sync();  // (not reached: the host launches this instance for C <= 256 only)
-  } else if (warp < 4 || g.epi2) {
+    else if constexpr (PCW > 4) run(IntC<8>{});  // (where PCW is 4 the host launches this instance for C <= 256 only)
+  } else {
+    // ================= epilogue warps, first job: the resident weights ===========================================
+    // Rows [rank * WR, +WR) of every channel tile of this group, expanded from the packed rows that wait in the activation
+    // buffers (the producers leave those alone until all are expanded).  A step takes 8 rows x 4 words, so that the 16-byte
+    // stores of a quarter-warp cover 8 consecutive rows of one 32-channel group, 128 contiguous bytes, and keeps three of
+    // them in flight (at 3x3 and C = 256 the third of a row: 12 words).  The first MMAs start when the first row of filter
+    // taps is there.  Against copying rows expanded beforehand (4x the bytes, 147 KB per CTA at most) the last weights of a
+    // 3x3, C = 256 CTA are in place after 7.5 k cycles instead of 10 k.
+    {
+      constexpr int BATCH = 3;
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
+      const int K64 = g.kh * g.kw * g.Cw;
+      const uint64_t* raw = reinterpret_cast<const uint64_t*>(a_s + g.raw_off);
+#pragma unroll 1
+      for (int item = warp < 4 ? warp : warp - 4; item < (thirds ? 3 * rb_n : rb_n); item += 8) {
+        const int j = (item >= rb_n ? 1 : 0) + (item >= 2 * rb_n ? 1 : 0), rb = item - j * rb_n;
+        const int k_lo = thirds ? K64 / 3 * j : 0, k_hi = thirds ? k_lo + K64 / 3 : K64;
+        const int row = rb * 8 + (lane & 7), r = row / WR, n = row % WR;  // row: of all resident rows of this CTA
+        const bool exists = (ng * g.nres + r) * NT + (int)rank * WR + n < g.O;  // (beyond O: zero weights)
+        const uint64_t* src = raw + row * K64;
+        uint8_t* dst = w_s + (size_t)(2 * r * K64 * WR + n) * 16;
+#pragma unroll 1
+        for (int k = k_lo + (lane >> 3); k < k_hi; k += 4 * BATCH) {
+          uint64_t word[BATCH];
+#pragma unroll
+          for (int u = 0; u < BATCH; u++) word[u] = k + 4 * u < k_hi ? src[k + 4 * u] : 0ull;
+#pragma unroll
+          for (int u = 0; u < BATCH; u++) {
+            if (k + 4 * u >= k_hi) break;
+            uint4 lo = expand32((uint32_t)word[u]), hi = expand32((uint32_t)(word[u] >> 32));
+            if (g.w_tail != ~0ull && (k + 4 * u) % g.Cw == g.Cw - 1) {  // (channel tails only)
+              lo = mask_channels(lo, (uint32_t)g.w_tail);
+              hi = mask_channels(hi, (uint32_t)(g.w_tail >> 32));
+            }
+            if (!exists) lo = hi = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u)) * WR * 16) = lo;
+            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u) + 1) * WR * 16) = hi;
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          arrive(bar_w_full + 8u * (uint32_t)j);
+          mbar_arrive(smem_u32(&bars[B_EXPANDED]));
+        }
+      }
+    }
+    if (warp < 4 || g.epi2) {
     // ================= epilogue warps: TMEM accumulator -> output ===============================================
+    chain_wait();
     uint32_t accb = 0, acc_phase = 0;  // accumulator of this round (one per tile and resident channel tile), parity of its uses
     bool failed = false;
     // with the second group, two warps share each quarter of the accumulator's rows: warps 0-3 take the even
@@ -979,6 +1033,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       in_flight--;
       if (++slot_u == (uint32_t)g.res_ring) { slot_u = 0; phase_u ^= 1u; }
     }
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (PAIR) cluster_sync_all();  // neither CTA leaves, or frees tensor memory, while the other may still use it
@@ -994,35 +1049,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   }
 }
 
-// Weights: packed bits [O][taps][Cw] -> e2m1 [blocks of 32 output channels][taps][C/32][32][16 bytes = 32 channels];
-// the blocks cover O rounded up to 128, rows beyond O are zero (e2m1 0.0: they contribute nothing).
-// Channels beyond C in the last 64-channel word (C not a multiple of 64) get 0.0 as well: whatever the activation rows
-// hold there, the product is 0 -- exactly as the zero tail bits of the packed words contribute nothing to Eq. 1.
-__global__ void tc_prepare_weights_kernel(const uint64_t* __restrict__ wp, int O, int C, int taps, int Cw, int cgroups,
-                                          long long units, uint4* __restrict__ out) {
-  const long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= units) return;
-  const int n = (int)(u & 31);
-  long long t = u >> 5;
-  const int grp = (int)(t % cgroups);
-  t /= cgroups;
-  const int tap = (int)(t % taps);
-  const int o = (int)(t / taps) * 32 + n;
-  uint4 bytes = make_uint4(0, 0, 0, 0);
-  if (o < O) {
-    const uint32_t half = (uint32_t)(wp[((long long)o * taps + tap) * Cw + (grp >> 1)] >> (32 * (grp & 1)));
-    bytes = expand32(half);
-    const int live = C - 32 * grp;  // channels of this group that exist
-    if (live < 32) {
-      // the validity bits go through the same expansion (and so the same channel order): 0xA marks a live nibble
-      const uint4 v = expand32(live <= 0 ? 0u : (1u << live) - 1u);
-      bytes.x &= ((v.x >> 3) & 0x11111111u) * 0xFu;
-      bytes.y &= ((v.y >> 3) & 0x11111111u) * 0xFu;
-      bytes.z &= ((v.z >> 3) & 0x11111111u) * 0xFu;
-      bytes.w &= ((v.w >> 3) & 0x11111111u) * 0xFu;
-    }
-  }
-  out[u] = bytes;
+// The prepared weights are the packed words at an address that bulk copies can start from.
+__global__ void tc_prepare_weights_kernel(const uint64_t* __restrict__ wp, long long words, uint64_t* __restrict__ out) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < words) out[t] = wp[t];
 }
 
 // 0: choose by size; 1: one CTA per tile; 2: CTA pairs wherever they are possible (environment DABNN_TC_MODE, read once).
@@ -1172,6 +1202,14 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   g.nacc = TC_ACC_COLS / g.ntile < TC_MAX_BUFS ? TC_ACC_COLS / g.ntile : TC_MAX_BUFS;
   size_t smem = wbytes + g.abufs * abytes + TC_SMEM_MISC;
   if (smem > (size_t)TC_SMEM_LIMIT) return DABNN_ERR_UNSUPPORTED;
+  {
+    // the packed rows wait for their expansion in the activation buffers: behind the first one where they fit (the first
+    // tile's activations are then expanded beside them), else in all of them
+    const size_t raw = wbytes / 4;
+    if (raw <= (g.abufs - 1) * abytes) { g.raw_off = (int)abytes; g.raw_first = 1; }
+    else if (raw <= g.abufs * abytes) { g.raw_off = 0; g.raw_first = 0; }
+    else return DABNN_ERR_UNSUPPORTED;
+  }
   g.res_ring = 0;
   if (EPI == EPI_BIREAL) {
     // The residual through a ring of bulk tensor copies, where shared memory has room for it beside every activation
@@ -1267,26 +1305,49 @@ void tc_plan(TcArgs& g, int O, int C, int taps) {
   if (nres > TC_MAX_RES) nres = TC_MAX_RES;
   if (nres > g.n_ntiles) nres = g.n_ntiles;
   const long long m_units = pair ? (g.m_tiles + 1) / 2 : g.m_tiles;
-  while (nres > 1 && (g.n_ntiles + nres - 1) / nres * m_units < (pair ? units2 : units1)) nres--;
   if (g.kgroups > 1) nres = 1;  // (the groups of a tile add up in one accumulator)
+  // How many of them: the units of a launch are dealt to groups of channel tiles first, so the busiest unit does
+  // ceil(m_units / (units / groups)) tiles of nres accumulators each.  Few resident tiles deal more evenly, many expand each
+  // activation tile fewer times; per accumulator the MMAs or the epilogue set the pace (cycles measured: 70 per MMA of 128
+  // columns, about 2000 for the epilogue), per tile the expansion does (600 + 200 per word), and a tile's hand-over costs
+  // some 400.  1x1, 128 -> 512 channels at 28x28, batch 16: 21.6 -> 15.1 us against "as many as leave every unit a tile".
+  const long long acc_cyc = (long long)taps * g.Cw * 70 > 2000 ? (long long)taps * g.Cw * 70 : 2000;
+  const long long exp_cyc = 600 + 200LL * g.Cw;
+  long long best = -1;
+  int best_n = 1;
+  for (int n = (int)nres; n >= 1; n--) {
+    const long long groups = (g.n_ntiles + n - 1) / n;
+    const long long per = (pair ? units2 : units1) / groups;  // units that share a group's tiles
+    if (per <= 0 && n > 1) continue;
+    const long long rounds = per > 0 ? (m_units + per - 1) / per : m_units;
+    const long long cost = rounds * ((n * acc_cyc > exp_cyc ? n * acc_cyc : exp_cyc) + 400) + n * wr * Kb / 256;
+    if (best < 0 || cost < best) {
+      best = cost;
+      best_n = n;
+    }
+  }
+  nres = best_n;
   g.nres = (int)nres;
   g.n_groups = (g.n_ntiles + g.nres - 1) / g.nres;
 }
 
-dabnn_status tc_fill(TcArgs& g, const uint64_t* a, dabnn_shape in, const void* w_tc, int O, dabnn_conv cv) {
-  if (!a || !w_tc) return DABNN_ERR_NULL;
+// w: packed words at a 16-byte boundary (a prepared buffer, or the caller's packed weights where they start on one)
+dabnn_status tc_fill(TcArgs& g, const uint64_t* a, dabnn_shape in, const void* w, int O, dabnn_conv cv) {
+  if (!a || !w) return DABNN_ERR_NULL;
   if (in.N <= 0 || in.C <= 0 || in.H <= 0 || in.W <= 0 || O <= 0) return DABNN_ERR_SHAPE;
   if (cv.kh <= 0 || cv.kw <= 0 || cv.stride_h <= 0 || cv.stride_w <= 0 || cv.pad_h < 0 || cv.pad_w < 0)
     return DABNN_ERR_SHAPE;
   if (cv.pad_value != 1 && cv.pad_value != -1) return DABNN_ERR_SHAPE;
-  if (!aligned(a, 8) || !aligned(w_tc, 16)) return DABNN_ERR_ALIGNMENT;
+  if (!aligned(a, 8) || !aligned(w, 16)) return DABNN_ERR_ALIGNMENT;
   const int OH = dabnn_out_dim(in.H, cv.kh, cv.stride_h, cv.pad_h), OW = dabnn_out_dim(in.W, cv.kw, cv.stride_w, cv.pad_w);
   if (OH <= 0 || OW <= 0) return DABNN_ERR_SHAPE;
   // what this engine covers; everything else is served by the xor/popcount kernel
   if (cv.stride_h != cv.stride_w || cv.stride_h > 2) return DABNN_ERR_UNSUPPORTED;
   if (!tc_covers(O, in.C, cv.kh * cv.kw)) return DABNN_ERR_UNSUPPORTED;
-  g.a = a; g.w_tc = static_cast<const uint8_t*>(w_tc);
-  g.N = in.N; g.H = in.H; g.W = in.W; g.Cw = (in.C + 63) / 64; g.C = tc_cpad(in.C);  // (the kernel sizes everything by whole words; see tc_prepare_weights_kernel)
+  g.a = a; g.w = static_cast<const uint64_t*>(w);
+  g.raw_off = g.raw_first = 0;
+  g.w_tail = in.C % 64 == 0 ? ~0ull : (1ull << (in.C % 64)) - 1;
+  g.N = in.N; g.H = in.H; g.W = in.W; g.Cw = (in.C + 63) / 64; g.C = tc_cpad(in.C);  // (the kernel sizes everything by whole words; see w_tail)
   g.O = O; g.kh = cv.kh; g.kw = cv.kw; g.ph = cv.pad_h; g.pw = cv.pad_w; g.OH = OH; g.OW = OW;
   g.S = cv.stride_h;
   // Stride 1 with pad <= k - 1: the slot grid keeps only the left and top padding of each image.  A tap that reaches the
@@ -1330,13 +1391,39 @@ bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv) {
   return 2 * (slots_total / 128) * tc_n_ntiles(O, nt) >= (long long)sm_count();  // measured: from half a wave of tiles on
 }
 
+// Packed-weight calls (epi: the output form) that run on this engine: where its estimated time is below that of the
+// xor/popcount kernel.  Both estimates are fits, in microseconds, to back-to-back launches on a B200 over 8 to 17 layer
+// shapes (C 16 to 512, 1x1 and 3x3, stride 1 and 2, O 16 to 2048) at batch 1 to 256:
+//   xor/popcount: 3.5 + 0.43 per million word multiply-adds + 0.9 per million outputs (+1.2 where a row is an odd number of
+//     words and is loaded in 8-byte pieces)
+//   tensor: 6 + up to 3 for expanding the resident weights (+3 at stride 2 with C > 128: one activation buffer, loaded after
+//     the weights) + 0.07 per million word multiply-adds + 0.9 per million outputs; outputs whose rows are not whole 32-byte
+//     pieces leave by 4-byte stores: +4 per million int32, +24 per million residual outputs
+// E.g. 3x3 with 256 channels at 14x14: batch 4 7.0 against 9.1 us, batch 8 8.6 / 9.1, batch 16 14.1 / 9.4, batch 64 42.0 / 12.4;
+// 64 channels at 56x56: batch 4 7.1 / 6.4, batch 64 60.5 / 20.2.
+bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi) {
+  if (cv.stride_h != cv.stride_w || cv.stride_h > 2 || !tc_covers(O, in.C, cv.kh * cv.kw)) return false;
+  const int taps = cv.kh * cv.kw, nt = tc_ntile(O, in.C, taps, false);
+  if (nt == 0) return false;
+  const double words = (in.C + 63) / 64;
+  const double outputs = (double)in.N * dabnn_out_dim(in.H, cv.kh, cv.stride_h, cv.pad_h) *
+                         dabnn_out_dim(in.W, cv.kw, cv.stride_w, cv.pad_w) * O * 1e-6;
+  const double macs = outputs * words * taps;
+  const double weights = (double)(O < nt ? O : nt) * tc_cpad(in.C) / 2 * taps / TC_WEIGHT_BUDGET;
+  const double t_int = 3.5 + 0.43 * macs + (((in.C + 63) / 64 * taps) % 2 ? 2.1 : 0.9) * outputs;
+  double t_tc = 6.0 + 3.0 * weights + 0.07 * macs + 0.9 * outputs;
+  if (cv.stride_h == 2 && in.C > 128) t_tc += 3.0;
+  if (O % 8 != 0) t_tc += (epi == EPI_I32 ? 4.0 : epi == EPI_BIREAL ? 24.0 : 0.0) * outputs;
+  return t_tc < t_int;
+}
+
 }  // namespace dabnn
 
 using namespace dabnn;
 
 extern "C" size_t dabnn_tc_weights_bytes(int O, int C, int kh, int kw) {
   if (O <= 0 || C <= 0 || kh <= 0 || kw <= 0 || !tc_covers(O, C, kh * kw)) return 0;
-  return (size_t)((O + 127) / 128 * 128) * kh * kw * (tc_cpad(C) / 2);
+  return (size_t)O * kh * kw * (tc_cpad(C) / 64) * 8;
 }
 
 extern "C" dabnn_status dabnn_tc_prepare_weights(const uint64_t* w_packed, int O, int C, int kh, int kw, void* w_tc,
@@ -1345,10 +1432,8 @@ extern "C" dabnn_status dabnn_tc_prepare_weights(const uint64_t* w_packed, int O
   if (O <= 0 || C <= 0 || kh <= 0 || kw <= 0) return DABNN_ERR_SHAPE;
   if (!tc_covers(O, C, kh * kw)) return DABNN_ERR_UNSUPPORTED;
   if (!aligned(w_packed, 8) || !aligned(w_tc, 16)) return DABNN_ERR_ALIGNMENT;
-  const int taps = kh * kw, cgroups = tc_cpad(C) / 32;
-  const long long units = (long long)((O + 127) / 128 * 128) * taps * cgroups;
-  tc_prepare_weights_kernel<<<ceil_div(units, 256), 256, 0, as_stream(stream)>>>(w_packed, O, C, taps, (C + 63) / 64, cgroups,
-                                                                                 units, static_cast<uint4*>(w_tc));
+  const long long words = (long long)O * kh * kw * (tc_cpad(C) / 64);
+  tc_prepare_weights_kernel<<<ceil_div(words, 256), 256, 0, as_stream(stream)>>>(w_packed, words, static_cast<uint64_t*>(w_tc));
   return launch_status();
 }
 
@@ -1379,6 +1464,37 @@ extern "C" dabnn_status dabnn_tc_bconv2d_bn_sign_pack(const uint64_t* a_packed, 
 }
 
 namespace dabnn {
+dabnn_status tc_bits_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv, int32_t* out,
+                             bool out_nchw, cudaStream_t st) {
+  TcArgs g;
+  dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
+  if (s != DABNN_OK) return s;
+  g.out = out;
+  g.out_nchw = out_nchw;
+  return tc_dispatch<EPI_I32>(g, st);
+}
+
+dabnn_status tc_bits_bn_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                  const float* scale, const float* shift, uint64_t* out_packed, cudaStream_t st) {
+  TcArgs g;
+  dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
+  if (s != DABNN_OK) return s;
+  g.scale = scale; g.shift = shift;
+  g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
+  return tc_dispatch<EPI_BNPACK>(g, st);
+}
+
+dabnn_status tc_bits_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                      const float* scale, const float* shift, const float* residual, float* y_out,
+                                      uint64_t* out_packed, cudaStream_t st) {
+  TcArgs g;
+  dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
+  if (s != DABNN_OK) return s;
+  g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;
+  g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
+  return tc_dispatch<EPI_BIREAL>(g, st);
+}
+
 dabnn_status tc_bireal_block(const uint64_t* a_packed, dabnn_shape in, const void* w_tc, int O, dabnn_conv cv,
                              const float* scale, const float* shift, const float* residual, float* y_out,
                              uint64_t* out_packed, bool chained, cudaStream_t st) {

@@ -21,6 +21,19 @@ inline int ceil_div(long long a, long long b) { return static_cast<int>((a + b -
 // (below that the integer-pipe kernel, which spreads small problems over many small CTAs, is faster).
 bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv);
 
+// Packed-weight calls (epi: 0 int32, 1 sign words, 2 residual stream) that are faster on the tensor-core engine.
+bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi);
+
+// The three output forms on the tensor-core engine from the caller's packed weights (16-byte aligned).  Arguments as of the
+// entry points of the same form, already checked; DABNN_ERR_UNSUPPORTED where the engine does not cover the layer.
+dabnn_status tc_bits_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv, int32_t* out,
+                             bool out_nchw, cudaStream_t st);
+dabnn_status tc_bits_bn_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                  const float* scale, const float* shift, uint64_t* out_packed, cudaStream_t st);
+dabnn_status tc_bits_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                      const float* scale, const float* shift, const float* residual, float* y_out,
+                                      uint64_t* out_packed, cudaStream_t st);
+
 // The Bi-Real block on the tensor-core engine as the forward launches it.  chained: with programmatic stream serialization
 // (the kernel sets itself up under its predecessor's tail; its weights and BN vectors must be constants of the stream).
 dabnn_status tc_bireal_block(const uint64_t* a_packed, dabnn_shape in, const void* w_tc, int O, dabnn_conv cv,

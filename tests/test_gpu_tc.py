@@ -402,3 +402,47 @@ def test_residual_ring_depths_in_a_child_process(ring):
     env = dict(os.environ, DABNN_TC_RES_RING=ring, PYTHONPATH=root + os.pathsep + os.environ.get("PYTHONPATH", ""))
     r = subprocess.run([sys.executable, "-c", _RING_SCRIPT], env=env, cwd=root, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "ring ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+# Packed-weight calls large enough for the route onto this engine (their CTAs expand the packed rows themselves): an odd
+# last word of a cut channel tile (O and K odd), a channel tail, no 3x3 thirds, CTA pairs with a cut tile, the rows staged
+# behind the first activation buffer or (stride 2) in the only one, channels in groups, several resident tiles, odd rows out.
+BITS_ROUTE_CASES = [
+    # N, C, H, W, O, k, pad, pad_value, stride
+    (60, 64, 28, 28, 65, 3, 1, -1, 1),
+    (40, 64, 28, 28, 33, 5, 2, +1, 1),
+    (130, 100, 27, 29, 70, 3, 1, +1, 2),
+    (64, 512, 7, 7, 450, 3, 1, -1, 1),
+    (200, 200, 14, 14, 130, 3, 1, -1, 2),
+    (30, 512, 14, 14, 1024, 1, 0, -1, 1),
+    (128, 1000, 14, 14, 96, 1, 0, -1, 1),
+    (30, 256, 14, 14, 256, 3, 1, -1, 1),
+    (24, 64, 56, 56, 64, 3, 1, -1, 1),
+]
+
+
+@pytest.mark.parametrize("case", BITS_ROUTE_CASES)
+def test_packed_weight_calls_on_this_engine_match_oracle(B, oracle_mod, case):
+    N, C, H, W, O, k, pad, pv, s = case
+    x, w = inputs(case)
+    o = oracle_mod
+    st = (s, s)
+    acc = o.bconv_bits(o.pack(x), C, o.pack_weights(w), st, (pad, pad), pv, o.NHWC)
+    rng = np.random.default_rng(O + N)
+    gamma, beta, mean, var = synth.bn_params(rng, O)
+    gamma[::3] *= -1.0
+    scale, shift = o.bn_fold(gamma, beta, mean, var)
+    res = (rng.standard_normal(acc.shape) * 15).astype(np.float32)
+    y, want_ybits = o.bn_add_sign_pack(acc, scale, shift, res)
+    want_bits = o.bn_sign_pack(acc, scale, shift)
+    a, wp = B.pack(dev(x)), B.pack_weights(dev(w))
+    off = torch.cat([wp.flatten()[:1], wp.flatten()])[1:].view(wp.shape)  # 8 bytes off a 16-byte boundary: the other engine
+    for weights in (wp, off):
+        assert np.array_equal(B.bconv2d(a, C, weights, st, (pad, pad), pv).cpu().numpy(), acc)
+        nchw = B.bconv2d(a, C, weights, st, (pad, pad), pv, out_layout=B.NCHW)
+        assert np.array_equal(nchw.cpu().numpy(), acc.transpose(0, 3, 1, 2))
+        assert np.array_equal(u64(B.bconv2d_bn_sign_pack(a, C, weights, dev(scale), dev(shift), st, (pad, pad), pv)), want_bits)
+        got_y, got_ybits = B.bconv2d_bn_add_sign_pack(a, C, weights, dev(scale), dev(shift), dev(res), st, (pad, pad), pv)
+        assert np.array_equal(got_y.cpu().numpy().view(np.uint32), y.view(np.uint32))
+        assert np.array_equal(u64(got_ybits), want_ybits)
+    assert B.last_device_flag() == 0
