@@ -97,6 +97,9 @@ dabnn_status dabnn_pack_weights(const float* w_oihw, int O, int C, int kh, int k
 
 /* Section 2.1.2, Eq. 1 -- binary convolution, int32 result.
  * a_packed: [N][H][W][Cw] for in = {N,C,H,W}; w_packed: [O][kh][kw][Cw];
+ * (These calls and the fused forms below run on the integer pipes or, where a launch is large enough to be faster there and
+ * w_packed is 16-byte aligned, on the tensor-core engine: same integers; see dabnn_last_device_flag for that engine's
+ * bounded waits, and dabnn_set_conv_variant / dabnn_set_conv_tile to keep a measurement on the integer pipes.)
  * out: int32, N*OH*OW*O elements in `out_layout` ([N][OH][OW][O] or [N][O][OH][OW]). */
 dabnn_status dabnn_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
                            int32_t* out, dabnn_layout out_layout, void* stream);
@@ -142,7 +145,7 @@ typedef struct {
   const float* down_shift[3];
   const float* fc_w;             /* fp32 [1000][512] */
   const float* fc_b;             /* fp32 [1000] */
-  const void* block_w_tc[16];    /* optional: weights expanded by dabnn_tc_prepare_weights, or NULL.  Where given and the
+  const void* block_w_tc[16];    /* optional: weights prepared by dabnn_tc_prepare_weights, or NULL.  Where given and the
                                     batch is large enough for the tensor-core engine to pay (all 16 blocks, stride 1 and
                                     stride 2, from about 70 images on; the early stages from 8), that engine runs the
                                     block; results are identical either way */
@@ -247,9 +250,10 @@ dabnn_status dabnn_binary_layer_host(const float* x_host, dabnn_shape in, const 
  * The Bi-Real epilogue of a long stride-1 launch whose rows are whole 128-byte chunks (O a multiple of 32, residual and
  * y_out 32-byte aligned) fetches the residual with bulk tensor copies; the library then encodes a tensor map on the host
  * in the call (cuTensorMapEncodeTiled, looked up through the runtime; if it is not there, ordinary loads are used).
- *   dabnn_tc_weights_bytes    bytes of the expanded weight buffer for a filter bank (0 = not covered): O rounded up to
- *                             128 rows of C*kh*kw/2 bytes, the same buffer for every launch form
- *   dabnn_tc_prepare_weights  w_packed [O][kh][kw][Cw] -> w_tc (device, 16-byte aligned, that many bytes); once per model
+ *   dabnn_tc_weights_bytes    bytes of the weight buffer of a filter bank on this engine (0 = not covered)
+ *   dabnn_tc_prepare_weights  w_packed [O][kh][kw][Cw] -> w_tc (device, 16-byte aligned, that many bytes); once per model.
+ *                             The buffer's content belongs to the library version that wrote it (at present the packed
+ *                             words: each CTA expands its own rows on chip)
  *   dabnn_tc_bconv2d*         as dabnn_bconv2d*, with w_tc in place of w_packed
  *   dabnn_tc_error_flag       synchronises nothing itself; copies the current device's error flag (1 if a bounded wait
  *                             inside a kernel ran out since the flag was last cleared, else 0; -1 if it cannot be read)
@@ -274,7 +278,7 @@ dabnn_status dabnn_tc_bconv2d_bn_sign_pack(const uint64_t* a_packed, dabnn_shape
 dabnn_status dabnn_tc_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const void* w_tc, int O,
                                                dabnn_conv cv, const float* scale, const float* shift, const float* residual,
                                                float* y_out, uint64_t* out_packed, void* stream);
-/* Eq. 1 (BGEMM) on the tensor-core engine: dabnn_bgemm with B expanded once by
+/* Eq. 1 (BGEMM) on the tensor-core engine: dabnn_bgemm with B prepared once by
  * dabnn_tc_prepare_weights(B, N, Kbits, 1, 1, b_tc) (dabnn_tc_weights_bytes(N, Kbits, 1, 1) bytes; Kbits <= 512).  Same integers. */
 dabnn_status dabnn_tc_bgemm(const uint64_t* A, int M, const void* b_tc, int N, int Kbits, int32_t* C, void* stream);
 int dabnn_tc_error_flag(void);
@@ -289,12 +293,13 @@ dabnn_status dabnn_tc_wait_expiry_selftest(const uint64_t* a_packed, dabnn_shape
 int dabnn_tc_set_max_ctas(int max_ctas);
 
 /* Selects the convolution inner loop for measurement runs: 0 = automatic (default),
- * 1 = one POPC per 32-bit word pair, 2 = carry-save (one POPC per two word pairs).  All give identical results.
+ * 1 = one POPC per 32-bit word pair, 2 = carry-save (one POPC per two word pairs); 1 and 2 keep every call on the integer
+ * pipes.  All give identical results.
  * Returns the previous setting.  Not thread-safe against concurrent calls into the library. */
 int dabnn_set_conv_variant(int variant);
 /* Forces the convolution's CTA tile for measurement runs: 0 = automatic (default), 1 = 128 pixels x 128 channels,
  * 2 = 128 x 64, 3 = 64 x 64, 4 = 32 x 32, 5 = 16 x 32 with all of K in flight (the choice for launches of less than
- * one wave).  All give identical results.  Returns the previous setting.
+ * one wave); every value but 0 keeps the calls on the integer pipes.  All give identical results.  Returns the previous setting.
  * (Environment, read once, for measurements: DABNN_CONV_POINTWISE=0 keeps long unpadded 1x1 stride-1 layers on the
  * one-tile-per-CTA kernel instead of the form that walks four pixel tiles with the weight rows resident.) */
 int dabnn_set_conv_tile(int tile);

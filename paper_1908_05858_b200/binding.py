@@ -471,7 +471,7 @@ def bireal18_forward_static(net: "Bireal18", images: torch.Tensor, logits: Optio
 
 # ---- tensor-core engine ---------------------------------------------------------------------------------------------
 class TcWeights:
-    """Expanded 4-bit (e2m1) weights for the tensor-core engine (dabnn_tc_prepare_weights), with the filter geometry."""
+    """Weights prepared for the tensor-core engine (dabnn_tc_prepare_weights), with the filter geometry."""
 
     def __init__(self, w_packed: torch.Tensor, C: int):
         w = _dev(w_packed, torch.int64, "w_packed")

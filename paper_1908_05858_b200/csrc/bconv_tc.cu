@@ -67,6 +67,7 @@ struct TcArgs {
   const uint64_t* w;   // packed weights [O][taps][Cw], 16-byte aligned
   uint64_t w_tail;     // the bits of a pixel's last word that are channels
   int raw_off;         // where a CTA's packed weight rows wait for their expansion, in bytes from the first activation buffer
+  int a_region;        // bytes of the activation buffers, or of the packed rows where those take more
   int raw_first;       // ... and the first fill of an activation buffer (0 or 1) that has to wait for it
   int N, H, W, Cw, C;
   int O, kh, kw, ph, pw, OH, OW;
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   const int a_bytes = KG ? g.slots * g.gw * 32 : g.slots * (g.C >> 1);  // bytes of one A buffer (one channel group)
   uint8_t* w_s = smem;                                   // [nres][taps][C/32][WR][16]
   uint8_t* a_s = smem + (size_t)g.nres * WR * Kb;        // [abufs][C/32][slots][16]
-  uint8_t* misc = a_s + (size_t)g.abufs * a_bytes;
+  uint8_t* misc = a_s + g.a_region;
   // [0..3] mma_done  [4..7] tmem_free  [8..11] a_full  [12..15] a_free  [16..18] w_full (thirds of the filter taps);
   // of a pair, the leader's tmem_free, a_full and w_full are used
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   if (g.chained) chain_trigger();  // the successor may start as CTAs of this launch leave (it waits for all of them itself)
   // Start-up, the roles side by side (a launch of one or two tiles per CTA is mostly this): warp 12 initialises the barriers
   // and requests the packed weight rows, warp 0 allocates tensor memory, all others derive the per-channel constants.
-  const bool thirds = g.kh == 3 && g.kw == 3;          // a 3x3 filter's weights become ready one row of taps at a time
+  const bool thirds = g.kh == 3 && g.kw == 3 && g.Cw > 2;  // a 3x3 filter's weights become ready one row of taps at a time
   const int rb_n = nres_here * (WR / 8);               // blocks of 8 weight rows of this CTA
   if (warp == 12) {
     if (lane == 0) {
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         if (k3) {
 #pragma unroll
           for (int t = 0; t < 9; t++) {
-            if (!KG && first && (t == 3 || t == 6) && !wait(smem_u32(&bars[B_W_FULL + t / 3]), 0)) *s_fail = 1;  // that row of taps
+            if (!KG && first && thirds && (t == 3 || t == 6) && !wait(smem_u32(&bars[B_W_FULL + t / 3]), 0)) *s_fail = 1;  // that row of taps
             const uint32_t a_lo = a_lo0 + off9[t];
 #pragma unroll
             for (int kb = 0; kb < KB; kb++)
@@ -503,7 +504,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       uint32_t ab = 0, a_phase = 0;  // A buffer of this tile and the parity of its `a_full` phase
       uint32_t accb = 0, acc_phase = 0;  // accumulator of this round and the parity of its uses so far
       int ar = 0;                    // accumulator rounds so far: one per (tile, resident channel tile)
-      bool ok = wait(smem_u32(&bars[B_W_FULL]), 0);  // first third of the resident weights (all of a filter that is not 3x3), and the scale factors
+      bool ok = wait(smem_u32(&bars[B_W_FULL]), 0);  // first third of the resident weights (or all of them), and the scale factors
       if (KG && thirds) ok = ok && wait(smem_u32(&bars[B_W_FULL + 1]), 0) && wait(smem_u32(&bars[B_W_FULL + 2]), 0);  // ... all of them
       if (!ok) *s_fail = 1;
       if constexpr (KG) {
@@ -652,7 +653,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     };
 
     {
-      // every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout (each warp: its quarter of the rows)
+      // every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout (each warp: its quarter of the rows).
+      // Here, before this role holds a tile's words in registers: after the first tile, or in the epilogue warps, it costs spills.
       const uint32_t one = 0x7F7F7F7Fu;
 #pragma unroll 1
       for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
@@ -716,55 +718,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     else if (g.Cw <= 4) run(IntC<4>{});
     else if constexpr (PCW > 4) run(IntC<8>{});  // (where PCW is 4 the host launches this instance for C <= 256 only)
   } else {
-    // ================= epilogue warps, first job: the resident weights ===========================================
-    // Rows [rank * WR, +WR) of every channel tile of this group, expanded from the packed rows that wait in the activation
-    // buffers (the producers leave those alone until all are expanded).  A step takes 8 rows x 4 words, so that the 16-byte
-    // stores of a quarter-warp cover 8 consecutive rows of one 32-channel group, 128 contiguous bytes, and keeps three of
-    // them in flight (at 3x3 and C = 256 the third of a row: 12 words).  The first MMAs start when the first row of filter
-    // taps is there.  Against copying rows expanded beforehand (4x the bytes, 147 KB per CTA at most) the last weights of a
-    // 3x3, C = 256 CTA are in place after 7.5 k cycles instead of 10 k.
-    {
-      constexpr int BATCH = 3;
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
-      const int K64 = g.kh * g.kw * g.Cw;
-      const uint64_t* raw = reinterpret_cast<const uint64_t*>(a_s + g.raw_off);
-#pragma unroll 1
-      for (int item = warp < 4 ? warp : warp - 4; item < (thirds ? 3 * rb_n : rb_n); item += 8) {
-        const int j = (item >= rb_n ? 1 : 0) + (item >= 2 * rb_n ? 1 : 0), rb = item - j * rb_n;
-        const int k_lo = thirds ? K64 / 3 * j : 0, k_hi = thirds ? k_lo + K64 / 3 : K64;
-        const int row = rb * 8 + (lane & 7), r = row / WR, n = row % WR;  // row: of all resident rows of this CTA
-        const bool exists = (ng * g.nres + r) * NT + (int)rank * WR + n < g.O;  // (beyond O: zero weights)
-        const uint64_t* src = raw + row * K64;
-        uint8_t* dst = w_s + (size_t)(2 * r * K64 * WR + n) * 16;
-#pragma unroll 1
-        for (int k = k_lo + (lane >> 3); k < k_hi; k += 4 * BATCH) {
-          uint64_t word[BATCH];
-#pragma unroll
-          for (int u = 0; u < BATCH; u++) word[u] = k + 4 * u < k_hi ? src[k + 4 * u] : 0ull;
-#pragma unroll
-          for (int u = 0; u < BATCH; u++) {
-            if (k + 4 * u >= k_hi) break;
-            uint4 lo = expand32((uint32_t)word[u]), hi = expand32((uint32_t)(word[u] >> 32));
-            if (g.w_tail != ~0ull && (k + 4 * u) % g.Cw == g.Cw - 1) {  // (channel tails only)
-              lo = mask_channels(lo, (uint32_t)g.w_tail);
-              hi = mask_channels(hi, (uint32_t)(g.w_tail >> 32));
-            }
-            if (!exists) lo = hi = make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u)) * WR * 16) = lo;
-            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u) + 1) * WR * 16) = hi;
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-          arrive(bar_w_full + 8u * (uint32_t)j);
-          mbar_arrive(smem_u32(&bars[B_EXPANDED]));
-        }
-      }
-    }
-    if (warp < 4 || g.epi2) {
-    // ================= epilogue warps: TMEM accumulator -> output ===============================================
-    chain_wait();
+    // ================= epilogue warps: the resident weights, then TMEM accumulator -> output =====================
+    const bool has_epi = warp < 4 || g.epi2;
     uint32_t accb = 0, acc_phase = 0;  // accumulator of this round (one per tile and resident channel tile), parity of its uses
     bool failed = false;
     // with the second group, two warps share each quarter of the accumulator's rows: warps 0-3 take the even
@@ -811,9 +766,58 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         if (++r_i >= nres_here) { r_i = 0; mt_i += mt_step; }
       }
     };
-    if (tma_res)
+    // (the ring's first requests go out before the weights are expanded, unless a previous kernel may still be writing there)
+    if (tma_res && has_epi && !g.chained)
       for (int i = 0; i < g.res_ring; i++) issue_next();
-    for (long long mt = mt_first; mt < mt_end && !failed; mt += mt_step) {
+    // Rows [rank * WR, +WR) of every channel tile of this group, expanded from the packed rows that wait in the activation
+    // buffers (the producers leave those alone until all are expanded).  A step takes 8 rows x 4 words, so that the 16-byte
+    // stores of a quarter-warp cover 8 consecutive rows of one 32-channel group, 128 contiguous bytes, and keeps three of
+    // them in flight (at 3x3 and C = 256 the third of a row: 12 words).  The first MMAs start when the first row of filter
+    // taps is there.  Against copying rows expanded beforehand (4x the bytes, 147 KB per CTA at most) the last weights of a
+    // 3x3, C = 256 CTA are in place after 7.5 k cycles instead of 10 k.
+    {
+      constexpr int BATCH = 3;
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
+      const int K64 = g.kh * g.kw * g.Cw;
+      const uint64_t* raw = reinterpret_cast<const uint64_t*>(a_s + g.raw_off);
+#pragma unroll 1
+      for (int item = warp < 4 ? warp : warp - 4; item < (thirds ? 3 * rb_n : rb_n); item += 8) {
+        const int j = (item >= rb_n ? 1 : 0) + (item >= 2 * rb_n ? 1 : 0), rb = item - j * rb_n;
+        const int k_lo = thirds ? K64 / 3 * j : 0, k_hi = thirds ? k_lo + K64 / 3 : K64;
+        const int row = rb * 8 + (lane & 7), r = row / WR, n = row % WR;  // row: of all resident rows of this CTA
+        const bool exists = (ng * g.nres + r) * NT + (int)rank * WR + n < g.O;  // (beyond O: zero weights)
+        const uint64_t* src = raw + row * K64;
+        uint8_t* dst = w_s + (size_t)(2 * r * K64 * WR + n) * 16;
+#pragma unroll 1
+        for (int k = k_lo + (lane >> 3); k < k_hi; k += 4 * BATCH) {
+          uint64_t word[BATCH];
+#pragma unroll
+          for (int u = 0; u < BATCH; u++) word[u] = k + 4 * u < k_hi ? src[k + 4 * u] : 0ull;
+#pragma unroll
+          for (int u = 0; u < BATCH; u++) {
+            if (k + 4 * u >= k_hi) break;
+            uint4 lo = expand32((uint32_t)word[u]), hi = expand32((uint32_t)(word[u] >> 32));
+            if (g.w_tail != ~0ull && (k + 4 * u) % g.Cw == g.Cw - 1) {  // (channel tails only)
+              lo = mask_channels(lo, (uint32_t)g.w_tail);
+              hi = mask_channels(hi, (uint32_t)(g.w_tail >> 32));
+            }
+            if (!exists) lo = hi = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u)) * WR * 16) = lo;
+            *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u) + 1) * WR * 16) = hi;
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          arrive(bar_w_full + 8u * (uint32_t)j);
+          mbar_arrive(smem_u32(&bars[B_EXPANDED]));
+        }
+      }
+    }
+    chain_wait();
+    if (tma_res && has_epi && g.chained)
+      for (int i = 0; i < g.res_ring; i++) issue_next();
+    for (long long mt = has_epi ? mt_first : mt_end; mt < mt_end && !failed; mt += mt_step) {
       const int row = 32 * (warp & 3) + lane;  // TMEM lane = slot row of the tile
       const uint32_t Q = (uint32_t)mt * 128u + (uint32_t)row;
       const uint32_t rr = fast_div(Q, g.magic_sp);
@@ -1033,7 +1037,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       in_flight--;
       if (++slot_u == (uint32_t)g.res_ring) { slot_u = 0; phase_u ^= 1u; }
     }
-    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (PAIR) cluster_sync_all();  // neither CTA leaves, or frees tensor memory, while the other may still use it
@@ -1205,10 +1208,12 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   {
     // the packed rows wait for their expansion in the activation buffers: behind the first one where they fit (the first
     // tile's activations are then expanded beside them), else in all of them
+    // (at least 78 KB are left beside the weights, and the packed rows are at most 36 KB)
     const size_t raw = wbytes / 4;
-    if (raw <= (g.abufs - 1) * abytes) { g.raw_off = (int)abytes; g.raw_first = 1; }
-    else if (raw <= g.abufs * abytes) { g.raw_off = 0; g.raw_first = 0; }
-    else return DABNN_ERR_UNSUPPORTED;
+    g.raw_first = raw <= (g.abufs - 1) * abytes ? 1 : 0;
+    g.raw_off = g.raw_first ? (int)abytes : 0;
+    g.a_region = (int)(raw > g.abufs * abytes ? raw : g.abufs * abytes);
+    smem += (size_t)g.a_region - g.abufs * abytes;
   }
   g.res_ring = 0;
   if (EPI == EPI_BIREAL) {
@@ -1394,13 +1399,14 @@ bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv) {
 // Packed-weight calls (epi: the output form) that run on this engine: where its estimated time is below that of the
 // xor/popcount kernel.  Both estimates are fits, in microseconds, to back-to-back launches on a B200 over 8 to 17 layer
 // shapes (C 16 to 512, 1x1 and 3x3, stride 1 and 2, O 16 to 2048) at batch 1 to 256:
-//   xor/popcount: 3.5 + 0.43 per million word multiply-adds + 0.9 per million outputs (+1.2 where a row is an odd number of
-//     words and is loaded in 8-byte pieces)
-//   tensor: 6 + up to 3 for expanding the resident weights (+3 at stride 2 with C > 128: one activation buffer, loaded after
-//     the weights) + 0.07 per million word multiply-adds + 0.9 per million outputs; outputs whose rows are not whole 32-byte
-//     pieces leave by 4-byte stores: +4 per million int32, +24 per million residual outputs
-// E.g. 3x3 with 256 channels at 14x14: batch 4 7.0 against 9.1 us, batch 8 8.6 / 9.1, batch 16 14.1 / 9.4, batch 64 42.0 / 12.4;
-// 64 channels at 56x56: batch 4 7.1 / 6.4, batch 64 60.5 / 20.2.
+//   xor/popcount: 3.5 + 0.43 per million word multiply-adds + 0.9 per million outputs (2.1 where a row is an odd number of
+//     words and is loaded in 8-byte pieces); the forms with sign words work on whole words of 64 channels
+//   tensor: 6 + up to 3 for expanding the resident weights + 0.07 per million word multiply-adds + 0.9 per million outputs
+//     (sign words 0.3); stride 2 +0.7, with C > 128 +2.3 more (one activation buffer, filled after the weights are expanded);
+//     the residual stream +1.5; outputs whose rows are not whole 32-byte pieces leave by 4-byte stores: +4 per million int32,
+//     +24 per million residual outputs
+// E.g. 3x3 with 256 channels at 14x14: batch 4 6.9 against 8.6 us, batch 8 8.6 / 8.7, batch 16 14.2 / 8.8, batch 64 42.0 / 11.5;
+// 64 channels at 56x56: batch 4 6.9 / 5.9, batch 64 51.6 / 17.1.
 bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi) {
   if (cv.stride_h != cv.stride_w || cv.stride_h > 2 || !tc_covers(O, in.C, cv.kh * cv.kw)) return false;
   const int taps = cv.kh * cv.kw, nt = tc_ntile(O, in.C, taps, false);
@@ -1410,9 +1416,11 @@ bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi) {
                          dabnn_out_dim(in.W, cv.kw, cv.stride_w, cv.pad_w) * O * 1e-6;
   const double macs = outputs * words * taps;
   const double weights = (double)(O < nt ? O : nt) * tc_cpad(in.C) / 2 * taps / TC_WEIGHT_BUDGET;
-  const double t_int = 3.5 + 0.43 * macs + (((in.C + 63) / 64 * taps) % 2 ? 2.1 : 0.9) * outputs;
-  double t_tc = 6.0 + 3.0 * weights + 0.07 * macs + 0.9 * outputs;
-  if (cv.stride_h == 2 && in.C > 128) t_tc += 3.0;
+  const double whole = epi == EPI_I32 ? 1.0 : (double)((O + 63) / 64 * 64) / O;
+  const double t_int = 3.5 + whole * (0.43 * macs + (((in.C + 63) / 64 * taps) % 2 ? 2.1 : 0.9) * outputs);
+  double t_tc = 6.0 + 3.0 * weights + 0.07 * macs + (epi == EPI_BNPACK ? 0.3 : 0.9) * outputs;
+  if (cv.stride_h == 2) t_tc += in.C > 128 ? 3.0 : 0.7;
+  if (epi == EPI_BIREAL) t_tc += 1.5;
   if (O % 8 != 0) t_tc += (epi == EPI_I32 ? 4.0 : epi == EPI_BIREAL ? 24.0 : 0.0) * outputs;
   return t_tc < t_int;
 }

@@ -418,6 +418,7 @@ BITS_ROUTE_CASES = [
     (128, 1000, 14, 14, 96, 1, 0, -1, 1),
     (30, 256, 14, 14, 256, 3, 1, -1, 1),
     (24, 64, 56, 56, 64, 3, 1, -1, 1),
+    (600, 64, 5, 5, 40, 11, 5, -1, 1),   # packed rows larger than all activation buffers
 ]
 
 
