@@ -67,7 +67,7 @@ struct TcArgs {
   const uint64_t* w;   // packed weights [O][taps][Cw], 16-byte aligned
   uint64_t w_tail;     // the bits of a pixel's last word that are channels
   int raw_off;         // where a CTA's packed weight rows wait for their expansion, in bytes from the first activation buffer
-  int a_region;        // bytes of the activation buffers, or of the packed rows where those take more
+  int misc_off;        // barriers and constants: behind the activation buffers (or the packed rows, where those take more)
   int raw_first;       // ... and the first fill of an activation buffer (0 or 1) that has to wait for it
   int N, H, W, Cw, C;
   int O, kh, kw, ph, pw, OH, OW;
@@ -244,6 +244,16 @@ __device__ __forceinline__ uint32_t acc_to_int(uint32_t acc_bits) {
   return __float_as_uint(__fadd_rn(__uint_as_float(acc_bits), 12582912.0f)) - 0x4B400000u;
 }
 
+// 16 consecutive columns of a warp's 32 accumulator rows.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 template <int V>
 struct IntC { static constexpr int value = V; };
 
@@ -255,7 +265,10 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t q, unsigned long long magi
 // KG: more channels than one activation buffer takes (C > 512, or > 256 at stride 2).  The weights stay resident; the
 // activations of a tile pass through the ring of activation buffers one channel group (g.gw words per row) at a time and
 // the MMAs of all groups add up in the same accumulator.  One channel tile per CTA, no CTA pairs.
-template <int NT, int EPI, int SPT, bool PAIR, bool RES_TMA = false, bool KG = false>
+// CWX: the words per pixel (C / 64) this instance is for, or 0 for any.  An instance for one count holds only that count's
+// MMA and expansion code, so that what its roles run lies close together: instruction fetches are a large part of the
+// stalls of a launch with few MMAs per tile.
+template <int NT, int EPI, int SPT, bool PAIR, bool RES_TMA = false, bool KG = false, int CWX = 0>
 __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_constant__ TcArgs g) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int WR = PAIR ? NT / 2 : NT;  // weight rows (output channels) of one channel tile held by this CTA
@@ -266,7 +279,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   const int a_bytes = KG ? g.slots * g.gw * 32 : g.slots * (g.C >> 1);  // bytes of one A buffer (one channel group)
   uint8_t* w_s = smem;                                   // [nres][taps][C/32][WR][16]
   uint8_t* a_s = smem + (size_t)g.nres * WR * Kb;        // [abufs][C/32][slots][16]
-  uint8_t* misc = a_s + g.a_region;
+  uint8_t* misc = smem + g.misc_off;
   // [0..3] mma_done  [4..7] tmem_free  [8..11] a_full  [12..15] a_free  [16..18] w_full (thirds of the filter taps);
   // of a pair, the leader's tmem_free, a_full and w_full are used
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
@@ -553,7 +566,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d_tmem = tmem_base + accb * (uint32_t)NT;
           const uint32_t b_base = b_lo0 + (uint32_t)r * b_tile;
-          switch (g.Cw) {  // C / 64 = 1..8
+          if constexpr (CWX != 0) issue_tile(d_tmem, a_lo0, b_base, a_step_t, ar == 0, 0u, IntC<CWX>{});
+          else switch (g.Cw) {  // C / 64 = 1..8
             case 1: issue_tile(d_tmem, a_lo0, b_base, a_step_t, ar == 0, 0u, IntC<1>{}); break;
             case 2: issue_tile(d_tmem, a_lo0, b_base, a_step_t, ar == 0, 0u, IntC<2>{}); break;
             case 3: issue_tile(d_tmem, a_lo0, b_base, a_step_t, ar == 0, 0u, IntC<3>{}); break;
@@ -712,7 +726,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       }
     };
     // C is a multiple of 64 up to 512: 1..8 words; the common counts get their own straight-line code
-    if constexpr (KG) run(IntC<PCW>{});  // groups of 8 words (4 where a thread holds five rows): g.gw == PCW
+    if constexpr (CWX != 0) run(IntC<CWX>{});
+    else if constexpr (KG) run(IntC<PCW>{});  // groups of 8 words (4 where a thread holds five rows): g.gw == PCW
     else if (g.Cw == 1) run(IntC<1>{});
     else if (g.Cw == 2) run(IntC<2>{});
     else if (g.Cw <= 4) run(IntC<4>{});
@@ -869,50 +884,51 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
             break;
           }
           in_flight--;
-          uint32_t v[32];
           const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(buf * NT + c0);
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-              "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-                "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-                "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-                "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-              : "r"(taddr));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           const int o = nt * NT + c0;
-          if (my_valid && o < g.O) {  // (O is a multiple of 32 on this path: a chunk exists whole or not at all)
-            const uint32_t src = ring0 + slot_u * TC_RING_CHUNK + srow * 128u;
-            float* yd = g.y_out + m * g.O + o;
-            uint32_t word = 0;
+          const bool live = my_valid && o < g.O;  // (O is a multiple of 32 on this path: a chunk exists whole or not at all)
+          const uint32_t src = ring0 + slot_u * TC_RING_CHUNK + srow * 128u;
+          float* yd = g.y_out + m * g.O + o;
+          uint32_t word = 0;
+          // (16 columns at a time in a rolled loop: the roles take turns on each scheduler, so straight-line code is fetched
+          // anew for every tile -- "no instruction" was the largest stall of this kernel, 2.4 of 10.8 cycles per issue)
+#pragma unroll 1
+          for (int p = 0; p < 2; p++) {
+            uint32_t v[16];
+            __syncwarp();
+            tmem_ld16(taddr + 16u * (uint32_t)p, v);
+            if (live) {
+              uint32_t half = 0;
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-              float rc[8], y[8];
+              for (int q = 0; q < 2; q++) {
+                float rc[8], y[8];
 #pragma unroll
-              for (int h = 0; h < 2; h++) {
-                const uint32_t ad = src + ((((uint32_t)(2 * q + h)) ^ (srow & 7u)) << 4);
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(rc[4 * h]), "=f"(rc[4 * h + 1]), "=f"(rc[4 * h + 2]), "=f"(rc[4 * h + 3])
-                             : "r"(ad));
-                const float4 sc = *reinterpret_cast<const float4*>(r_scale + c0 + 8 * q + 4 * h);
-                const float4 sh = *reinterpret_cast<const float4*>(r_shift + c0 + 8 * q + 4 * h);
-                y[4 * h] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h]), sc.x, sh.x);
-                y[4 * h + 1] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 1]), sc.y, sh.y);
-                y[4 * h + 2] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 2]), sc.z, sh.z);
-                y[4 * h + 3] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 3]), sc.w, sh.w);
+                for (int h = 0; h < 2; h++) {
+                  const uint32_t ad = src + ((((uint32_t)(4 * p + 2 * q + h)) ^ (srow & 7u)) << 4);
+                  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                               : "=f"(rc[4 * h]), "=f"(rc[4 * h + 1]), "=f"(rc[4 * h + 2]), "=f"(rc[4 * h + 3])
+                               : "r"(ad));
+                  const float4 sc = *reinterpret_cast<const float4*>(r_scale + c0 + 16 * p + 8 * q + 4 * h);
+                  const float4 sh = *reinterpret_cast<const float4*>(r_shift + c0 + 16 * p + 8 * q + 4 * h);
+                  y[4 * h] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h]), sc.x, sh.x);
+                  y[4 * h + 1] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 1]), sc.y, sh.y);
+                  y[4 * h + 2] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 2]), sc.z, sh.z);
+                  y[4 * h + 3] = __fmaf_rn(__uint_as_float(v[8 * q + 4 * h + 3]), sc.w, sh.w);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                  y[j] = __fadd_rn(y[j], rc[j]);
+                  half |= (uint32_t)(y[j] < 0.0f) << (8 * q + j);
+                }
+                st_global_v8(yd + 16 * p + 8 * q, __float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]),
+                             __float_as_uint(y[3]), __float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]),
+                             __float_as_uint(y[7]));
               }
-#pragma unroll
-              for (int j = 0; j < 8; j++) {
-                y[j] = __fadd_rn(y[j], rc[j]);
-                word |= (uint32_t)(y[j] < 0.0f) << (8 * q + j);
-              }
-              st_global_v8(yd + 8 * q, __float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]), __float_as_uint(y[3]),
-                           __float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]), __float_as_uint(y[7]));
+              word |= half << (16 * p);
             }
-            if (g.out_packed32 != nullptr) g.out_packed32[m * g.Ow32 + (o >> 5)] = word;
-          } else if (my_valid && o < g.Ow32 * 32 && g.out_packed32 != nullptr) {
-            g.out_packed32[m * g.Ow32 + (o >> 5)] = 0u;  // sign words are written whole: the half beyond O holds zeros
           }
+          // (sign words are written whole: a half beyond O holds zeros)
+          if (my_valid && o < g.Ow32 * 32 && g.out_packed32 != nullptr) g.out_packed32[m * g.Ow32 + (o >> 5)] = word;
           // the chunk is in registers (or stored): its buffer takes the next request
           if (++slot_u == (uint32_t)g.res_ring) { slot_u = 0; phase_u ^= 1u; }
           __syncwarp();
@@ -1090,9 +1106,9 @@ int tc_ntile(int O, int C, int taps, bool pair) {
 // Channel tiles cover O rounded up to whole 64-bit sign words (rows beyond O hold zero weights).
 int tc_n_ntiles(int O, int nt) { return ((O + 63) / 64 * 64 + nt - 1) / nt; }
 
-template <int NT, int EPI, int SPT, bool PAIR, bool RES_TMA = false, bool KG = false>
+template <int NT, int EPI, int SPT, bool PAIR, bool RES_TMA = false, bool KG = false, int CWX = 0>
 dabnn_status tc_launch(const TcArgs& g, size_t smem, cudaStream_t st) {
-  auto kern = bconv_tc_kernel<NT, EPI, SPT, PAIR, RES_TMA, KG>;
+  auto kern = bconv_tc_kernel<NT, EPI, SPT, PAIR, RES_TMA, KG, CWX>;
   static bool configured[kMaxDevices] = {};
   static int max_units_dev[kMaxDevices] = {};  // CTAs (pairs) that can be resident at once
   const int dev = current_device();
@@ -1212,8 +1228,9 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
     const size_t raw = wbytes / 4;
     g.raw_first = raw <= (g.abufs - 1) * abytes ? 1 : 0;
     g.raw_off = g.raw_first ? (int)abytes : 0;
-    g.a_region = (int)(raw > g.abufs * abytes ? raw : g.abufs * abytes);
-    smem += (size_t)g.a_region - g.abufs * abytes;
+    const size_t region = raw > g.abufs * abytes ? raw : g.abufs * abytes;
+    g.misc_off = (int)(wbytes + region);
+    smem += region - g.abufs * abytes;
   }
   g.res_ring = 0;
   if (EPI == EPI_BIREAL) {
@@ -1235,8 +1252,9 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   }
   if constexpr (EPI == EPI_BIREAL && !PAIR) {
     if (g.res_ring > 0) {
-      if (g.ntile == 128) return tc_launch<128, EPI, 2, false, true>(g, smem, st);
-      return tc_launch<64, EPI, 2, false, true>(g, smem, st);
+      if (g.ntile == 128)
+        return g.Cw == 2 ? tc_launch<128, EPI, 2, false, true, false, 2>(g, smem, st) : tc_launch<128, EPI, 2, false, true>(g, smem, st);
+      return g.Cw == 1 ? tc_launch<64, EPI, 2, false, true, false, 1>(g, smem, st) : tc_launch<64, EPI, 2, false, true>(g, smem, st);
     }
   }
   if constexpr (!PAIR) {
