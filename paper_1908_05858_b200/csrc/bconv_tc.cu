@@ -1211,6 +1211,22 @@ bool tc_residual_map(CUtensorMap* map, const float* residual, long long pixels, 
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The instance for the layer's word count where there is one (64, 128, 256 and 512 channels), else the one for any count.
+template <int NT, int EPI, int SPT, bool PAIR>
+dabnn_status tc_launch_words(const TcArgs& g, size_t smem, cudaStream_t st) {
+  if constexpr (PAIR) {
+    if (NT == 128 && SPT == 2 && g.Cw == 8) return tc_launch<128, EPI, 2, true, false, false, 8>(g, smem, st);
+  } else if constexpr (NT == 128 || SPT == 2) {
+    switch (g.Cw) {
+      case 1: return tc_launch<NT, EPI, SPT, false, false, false, 1>(g, smem, st);
+      case 2: if constexpr (NT == 128) return tc_launch<NT, EPI, SPT, false, false, false, 2>(g, smem, st); break;
+      case 4: if constexpr (NT == 128) return tc_launch<NT, EPI, SPT, false, false, false, 4>(g, smem, st); break;
+      case 8: if constexpr (NT == 128 && SPT == 2) return tc_launch<NT, EPI, SPT, false, false, false, 8>(g, smem, st); break;
+    }
+  }
+  return tc_launch<NT, EPI, SPT, PAIR>(g, smem, st);
+}
+
 template <int EPI, bool PAIR>
 dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   const size_t wr = (size_t)g.ntile / (PAIR ? 2 : 1);
@@ -1277,13 +1293,13 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   }
   if (g.slots <= 256) {
     switch (g.ntile) {
-      case 128: return tc_launch<128, EPI, 2, PAIR>(g, smem, st);
-      case 64: return tc_launch<64, EPI, 2, PAIR>(g, smem, st);
+      case 128: return tc_launch_words<128, EPI, 2, PAIR>(g, smem, st);
+      case 64: return tc_launch_words<64, EPI, 2, PAIR>(g, smem, st);
       case 32: if constexpr (!PAIR) return tc_launch<32, EPI, 2, false>(g, smem, st);
     }
   } else if (g.Cw <= 4) {
     switch (g.ntile) {
-      case 128: return tc_launch<128, EPI, TC_MAX_SPT, PAIR>(g, smem, st);
+      case 128: return tc_launch_words<128, EPI, TC_MAX_SPT, PAIR>(g, smem, st);
       case 64: return tc_launch<64, EPI, TC_MAX_SPT, PAIR>(g, smem, st);
       case 32: if constexpr (!PAIR) return tc_launch<32, EPI, TC_MAX_SPT, false>(g, smem, st);
     }
