@@ -41,6 +41,9 @@ PACK_SHAPES = [
     (4, 512, 7, 7),     # tile path: H*W = 49
     (2, 100, 15, 13),   # tile path, two pixel tiles, channel tail
     (1, 2100, 3, 3),    # more than 32 words: generic path
+    (3, 100, 15, 15),   # whole-image path: H*W = 225, channel tail, a run of 36 * 225 values
+    (2, 68, 1, 3),      # whole-image path with four channels in the last word
+    (70, 512, 7, 7),    # whole-image path, many CTAs
 ]
 
 
@@ -55,7 +58,11 @@ def test_pack_nchw(B, oracle_mod, shape):
     assert np.array_equal(got, oracle_mod.pack(x, oracle_mod.NCHW))
 
 
-@pytest.mark.parametrize("shape", [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (1, 3, 3, 4), (4, 31, 17, 128)])
+# (after the first five: the flat-bitmap path -- a last vector of one to three values, several pixel tiles,
+# large tiles, the largest C of the path and one beyond it)
+@pytest.mark.parametrize("shape", [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (1, 3, 3, 4), (4, 31, 17, 128), (1, 1, 1, 1),
+                                   (3, 1, 1, 1), (1, 7, 11, 35), (2, 33, 17, 33), (37, 27, 29, 100), (90, 28, 28, 70), (1, 6, 6, 4090),
+                                   (1, 3, 3, 4099)])
 def test_pack_nhwc(B, oracle_mod, shape):
     rng = np.random.default_rng(sum(shape) + 1)
     x = rng.standard_normal(shape).astype(np.float32)
