@@ -146,8 +146,8 @@ typedef struct {
   const float* fc_w;             /* fp32 [1000][512] */
   const float* fc_b;             /* fp32 [1000] */
   const void* block_w_tc[16];    /* optional: weights prepared by dabnn_tc_prepare_weights, or NULL.  Where given and the
-                                    batch is large enough for the tensor-core engine to pay (all 16 blocks, stride 1 and
-                                    stride 2, from about 70 images on; the early stages from 8), that engine runs the
+                                    layer is large enough to be faster on the tensor-core engine
+                                    (the early stages from 4 images, all blocks from about 64), that engine runs the
                                     block; results are identical either way */
 } dabnn_bireal18_params;
 

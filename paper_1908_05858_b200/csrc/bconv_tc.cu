@@ -1420,16 +1420,6 @@ dabnn_status tc_fill(TcArgs& g, const uint64_t* a, dabnn_shape in, const void* w
 
 }  // namespace
 
-bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv) {
-  if (cv.stride_h != cv.stride_w || cv.stride_h > 2 || !tc_covers(O, in.C, cv.kh * cv.kw)) return false;
-  const int nt = tc_ntile(O, in.C, cv.kh * cv.kw, false);
-  if (nt == 0) return false;
-  const int S = cv.stride_h;
-  const int pads = (S == 1 && cv.pad_h <= cv.kh - 1 && cv.pad_w <= cv.kw - 1) ? 1 : 2;  // as in tc_fill
-  const long long slots_total = (long long)in.N * ((in.H + pads * cv.pad_h + S - 1) / S) * ((in.W + pads * cv.pad_w + S - 1) / S);
-  return 2 * (slots_total / 128) * tc_n_ntiles(O, nt) >= (long long)sm_count();  // measured: from half a wave of tiles on
-}
-
 // Packed-weight calls (epi: the output form) that run on this engine: where its estimated time is below that of the
 // xor/popcount kernel.  Both estimates are fits, in microseconds, to back-to-back launches on a B200 over 8 to 17 layer
 // shapes (C 16 to 512, 1x1 and 3x3, stride 1 and 2, O 16 to 2048) at batch 1 to 256:
@@ -1441,7 +1431,7 @@ bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv) {
 //     +24 per million residual outputs
 // E.g. 3x3 with 256 channels at 14x14: batch 4 6.9 against 8.6 us, batch 8 8.6 / 8.7, batch 16 14.2 / 8.8, batch 64 42.0 / 11.5;
 // 64 channels at 56x56: batch 4 6.9 / 5.9, batch 64 51.6 / 17.1.
-bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi) {
+bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi, double hidden) {
   if (cv.stride_h != cv.stride_w || cv.stride_h > 2 || !tc_covers(O, in.C, cv.kh * cv.kw)) return false;
   const int taps = cv.kh * cv.kw, nt = tc_ntile(O, in.C, taps, false);
   if (nt == 0) return false;
@@ -1456,7 +1446,7 @@ bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi) {
   if (cv.stride_h == 2) t_tc += in.C > 128 ? 3.0 : 0.7;
   if (epi == EPI_BIREAL) t_tc += 1.5;
   if (O % 8 != 0) t_tc += (epi == EPI_I32 ? 4.0 : epi == EPI_BIREAL ? 24.0 : 0.0) * outputs;
-  return t_tc < t_int;
+  return t_tc - hidden < t_int;
 }
 
 }  // namespace dabnn

@@ -41,20 +41,6 @@ __host__ __device__ constexpr int stem_half(int ps) {
   return h;
 }
 
-// Two fp32 fused multiply-adds in one instruction (fma.rn.f32x2): each lane of the pair is the same correctly rounded
-// fmaf as the scalar instruction, so results do not change; it halves the issue slots of an FMA-bound loop.
-__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void fma_f32x2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 template <int TS, int PPT, int CPT>
 __global__ void __launch_bounds__((TS * TS / PPT) * 4, 2) stem_conv_bn(const float* __restrict__ img,
                                                                        const float* __restrict__ w,
@@ -886,10 +872,10 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
 
   dabnn_status s;
   if (sm) {
-    // the stem output area holds the module's three scratch tensors: s1 (half of it), a1 and the concatenation (a quarter each)
-    float* a1 = stem_out + (size_t)N * 112 * 112 * 32;
+    // the stem output area holds the module's two scratch tensors: a1 and the concatenation
+    float* a1 = stem_out;
     float* cat = a1 + (size_t)N * 112 * 112 * 16;
-    if ((s = launch_stem_module(sm, images, N, stem_out, a1, cat, cur, bits_in, st)) != DABNN_OK) return s;
+    if ((s = launch_stem_module(sm, images, N, a1, cat, cur, bits_in, st)) != DABNN_OK) return s;
   } else {
     s = (N * 49 >= 2 * sm_count()) ? launch_stem_8x8(p, images, N, stem_out, st)
                                    : (N == 1 ? launch_stem<8, 2, 8>(p, images, N, stem_out, st)  // one image: 392 half-tile CTAs
@@ -929,7 +915,10 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
     const int stride = down ? 2 : 1;
     const dabnn_conv cv = {3, 3, stride, stride, 1, 1, -1};
     s = DABNN_ERR_UNSUPPORTED;
-    if (p->block_w_tc[b] != nullptr && tc_worthwhile(in, O, cv))  // tensor-core engine where it covers the layer and pays
+    // tensor-core engine where it covers the layer and pays; chained launches hide part of its start-up (measured: a credit
+    // of 1.5 us against lone launches; batch 8 240 -> 234 us, batch 12 283 -> 269, batch 16 340 -> 322, batch 4 unchanged;
+    // with 3 us batch 2 and 4 lose 3 us each)
+    if (p->block_w_tc[b] != nullptr && tc_bits_worthwhile(in, O, cv, 2, tc_chain ? 1.5 : 0.0))
       s = tc_bireal_block(bits_in, in, p->block_w_tc[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
                           b == 15 ? nullptr : bits_out, tc_chain, st);
     if (s == DABNN_ERR_UNSUPPORTED)

@@ -17,12 +17,9 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 inline int ceil_div(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
 
-// True when the tensor-core engine covers this layer AND the layer has enough pixel tiles for at least half of the SMs
-// (below that the integer-pipe kernel, which spreads small problems over many small CTAs, is faster).
-bool tc_worthwhile(dabnn_shape in, int O, dabnn_conv cv);
-
-// Packed-weight calls (epi: 0 int32, 1 sign words, 2 residual stream) that are faster on the tensor-core engine.
-bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi);
+// Layers (epi: 0 int32, 1 sign words, 2 residual stream) that are faster on the tensor-core engine than on the integer pipes;
+// hidden: microseconds of its start-up that pass under a previous kernel.
+bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi, double hidden = 0.0);
 
 // The three output forms on the tensor-core engine from the caller's packed weights (16-byte aligned).  Arguments as of the
 // entry points of the same form, already checked; DABNN_ERR_UNSUPPORTED where the engine does not cover the layer.
@@ -60,6 +57,20 @@ __device__ __forceinline__ float4 ld_nc_f4(const float* p) {
   return v;
 }
 
+// Two fp32 fused multiply-adds in one instruction (fma.rn.f32x2): each lane of the pair is the same correctly rounded
+// fmaf as the scalar instruction, so results do not change; it halves the issue slots of an FMA-bound loop.
+__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma_f32x2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
 template <typename... KArgs, typename... Args>
 inline void launch_chain(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   if (!g_chain_launch) {
@@ -81,8 +92,8 @@ inline void launch_chain(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
 #endif
 
 // The STEM module front end of Bi-Real Net 18 (stem_module.cu): fp32 [N][56][56][64] and its packed signs from the images.
-dabnn_status launch_stem_module(const dabnn_stem_module_params* sm, const float* images, int N, float* s1, float* a1,
-                                float* cat, float* out, uint64_t* bits, cudaStream_t st);
+dabnn_status launch_stem_module(const dabnn_stem_module_params* sm, const float* images, int N, float* a1, float* cat,
+                                float* out, uint64_t* bits, cudaStream_t st);
 
 // Per-device host caches (function attributes set, SM counts, symbol addresses) are arrays over the device ordinal.
 constexpr int kMaxDevices = 64;
