@@ -273,6 +273,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int WR = PAIR ? NT / 2 : NT;  // weight rows (output channels) of one channel tile held by this CTA
   constexpr uint32_t PEERS = PAIR ? 2 : 1;
+  // Sign words with two epilogue groups: each group takes every other accumulator whole, so that a lane holds the four words
+  // of its row's 128 channels and stores them as one 16-byte piece instead of four 4-byte ones.  1x1, 512 -> 2048 channels at
+  // 14x14, batch 256, with its pack: 79.9 -> 75.1 us.
+  constexpr bool ALTERNATE = EPI == EPI_BNPACK && NT == 128;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // 0: the CTA that issues the pair's MMAs
   const int Kb = g.kh * g.kw * (g.C >> 1);               // bytes per weight row
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     if (lane == 0) {
       for (int i = 0; i < TC_MAX_BUFS; i++) {
         mbar_init(smem_u32(&bars[B_MMA_DONE + i]), 1);
-        mbar_init(smem_u32(&bars[B_TMEM_FREE + i]), (g.epi2 ? 8 : 4) * PEERS);  // one arrival per epilogue warp
+        mbar_init(smem_u32(&bars[B_TMEM_FREE + i]), (g.epi2 && !ALTERNATE ? 8 : 4) * PEERS);  // one arrival per epilogue warp of a round
         mbar_init(smem_u32(&bars[B_A_FULL + i]), 4 * PEERS + (uint32_t)g.extra_arrivals);  // one arrival per producer warp
         mbar_init(smem_u32(&bars[B_A_FREE + i]), 1);
       }
@@ -739,8 +743,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     bool failed = false;
     // with the second group, two warps share each quarter of the accumulator's rows: warps 0-3 take the even
     // 32-column chunks, warps 8-11 the odd ones
-    const int c_first = warp >= 8 ? 32 : 0;
-    const int c_step = g.epi2 ? 64 : 32;
+    const int c_first = warp >= 8 && !ALTERNATE ? 32 : 0;
+    const int c_step = g.epi2 && !ALTERNATE ? 64 : 32;
+    uint32_t round = warp >= 8 ? 1u : 0u;  // (ALTERNATE) even: this group's accumulator
+    const bool wide_bits = ALTERNATE && (g.Ow32 & 3) == 0 && (reinterpret_cast<uintptr_t>(g.out_packed32) & 15) == 0;
     const uint64_t pol_stream = EPI == EPI_I32 ? evict_first_policy() : 0ull;  // (made once, not per store)
     // The residual as bulk tensor copies (g.res_ring > 0): every epilogue warp owns a ring of 4 KB chunks (32 rows x 32
     // channels) and its lane 0 requests the chunks in the order the warp will use them, `res_ring` chunks ahead -- across
@@ -848,6 +854,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       const bool wide_y = EPI == EPI_BIREAL && (g.O & 7) == 0 &&
                           ((reinterpret_cast<uintptr_t>(g.residual) | reinterpret_cast<uintptr_t>(g.y_out)) & 31) == 0;
       for (int r = 0; r < nres_here; r++) {
+      if (ALTERNATE && g.epi2 && (round++ & 1u)) {  // the other group's
+        if (++accb == (uint32_t)g.nacc) { accb = 0; acc_phase ^= 1u; }
+        continue;
+      }
+      uint4 row_words = make_uint4(0, 0, 0, 0);
       const uint32_t buf = accb;
       const int nt = ng * g.nres + r;  // this round's channel tile
       const float* r_scale = s_scale + r * NT;
@@ -996,7 +1007,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
           }
           word ^= reinterpret_cast<const uint32_t*>(s_shift)[(r * NT + c0) >> 5];
           word &= nch >= 32 ? 0xFFFFFFFFu : (nch > 0 ? (1u << nch) - 1u : 0u);  // channels beyond O: bit 0
-          g.out_packed32[m * g.Ow32 + (o >> 5)] = word;
+          if (wide_bits) {  // (whole 128-channel rows: every chunk of the tile passes here)
+            if (c0 == 0) row_words.x = word;
+            else if (c0 == 32) row_words.y = word;
+            else if (c0 == 64) row_words.z = word;
+            else {
+              row_words.w = word;
+              *reinterpret_cast<uint4*>(g.out_packed32 + m * g.Ow32 + ((o - 96) >> 5)) = row_words;
+            }
+          } else {
+            g.out_packed32[m * g.Ow32 + (o >> 5)] = word;
+          }
         } else {
           if (o >= g.Ow32 * 32) continue;  // sign words are written whole (tail bits 0), nothing beyond them
           float y[32];
