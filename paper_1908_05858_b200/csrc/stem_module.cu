@@ -14,110 +14,6 @@ namespace dabnn {
 
 namespace {
 
-// Direct fp32 convolution, zero padding, then y = fmaf(acc, scale, shift) and an optional ReLU, as a register-tiled product
-// with a fixed summation order.  A CTA of 256 threads owns 128 consecutive output pixels x BN output channels; K = CIN * k * k
-// is walked in chunks of CG channels x all taps (k index = c * taps + tap ascending: the pinned order).  Per chunk the
-// im2col values of the CTA's pixels go to shared memory k-major ([k][pixel]: a thread later reads its 4 pixels as one
-// 128-bit load) and the filters as [k][channel] (broadcast reads); thread (tx, ty) keeps 4 pixels x TN = BN / 8 channels.
-// The loader thread of pixel p fetches CG consecutive channels of a tap with one vector load.  Taps outside the image are
-// zeros: fmaf(0, w, acc) = acc.
-// x: NHWC with CIN channels per pixel; y: NHWC with y_stride channels per pixel, written at channel y_off.
-template <int K, int S, int PAD, int CIN, int BN, int CG, bool RELU>
-__global__ void __launch_bounds__(256) conv_fp32_pinned(const float* __restrict__ x, int N, int H, int W, int OH, int OW,
-                                                        const float* __restrict__ w_oihw, const float* __restrict__ scale,
-                                                        const float* __restrict__ shift, float* __restrict__ y,
-                                                        int y_stride, int y_off) {
-  constexpr int BM = 128, T = K * K, KC = CG * T, TN = BN / 8, AP = BM + 4, WP = BN + 4;
-  static_assert(CIN % CG == 0 && BN % 16 == 0 && (K == 1 ? CG % 8 == 0 : CG == 4), "tile");
-  __shared__ __align__(16) float a_s[KC * AP];
-  __shared__ __align__(16) float w_s[KC * WP];
-  const int tid = threadIdx.x;
-  const long long npix = (long long)N * OH * OW;
-  const long long p0 = (long long)blockIdx.x * BM;
-  const int o0 = blockIdx.y * BN;
-  // loader role: pixel lp, and one half of the chunk's taps (or channels, for a single tap)
-  const int lp = tid & (BM - 1), lhalf = tid >> 7;
-  const long long pl = p0 + lp;
-  int ih0 = 0, iw0 = 0;
-  long long xn = -1;  // offset of image n in x, or -1 for a pixel beyond the end
-  if (pl < npix) {
-    const int ow = (int)(pl % OW), oh = (int)((pl / OW) % OH);
-    const long long n = pl / ((long long)OW * OH);
-    ih0 = oh * S - PAD;
-    iw0 = ow * S - PAD;
-    xn = n * (long long)CIN * H * W;
-  }
-  const int tx = tid & 31, ty = tid >> 5;
-  float acc[4][TN];
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < TN; j++) acc[i][j] = 0.0f;
-
-  for (int c0 = 0; c0 < CIN; c0 += CG) {
-    // filters of this chunk: w_s[k][o] = w[o0 + o][c0 * T + k]
-    for (int idx = tid; idx < KC * BN; idx += 256) {
-      const int o = idx / KC, k = idx - o * KC;  // consecutive threads: consecutive k of one filter (contiguous in OIHW)
-      w_s[k * WP + o] = w_oihw[(size_t)(o0 + o) * (CIN * T) + c0 * T + k];
-    }
-    // im2col values of this chunk
-    if (T == 1) {
-      // one tap: the two loader threads of a pixel take half of the chunk's channels each
-#pragma unroll
-      for (int q = 0; q < CG / 8; q++) {
-        const int cc = lhalf * (CG / 2) + 4 * q;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (xn >= 0) v = __ldg(reinterpret_cast<const float4*>(x + xn + ((long long)ih0 * W + iw0) * CIN + c0 + cc));
-        a_s[(cc + 0) * AP + lp] = v.x; a_s[(cc + 1) * AP + lp] = v.y; a_s[(cc + 2) * AP + lp] = v.z; a_s[(cc + 3) * AP + lp] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int t = 0; t < T; t++) {
-        if ((t & 1) != lhalf) continue;
-        const int ih = ih0 + t / K, iw = iw0 + t % K;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (xn >= 0 && ih >= 0 && ih < H && iw >= 0 && iw < W) v = __ldg(reinterpret_cast<const float4*>(x + xn + ((long long)ih * W + iw) * CIN + c0));
-        a_s[(0 * T + t) * AP + lp] = v.x; a_s[(1 * T + t) * AP + lp] = v.y; a_s[(2 * T + t) * AP + lp] = v.z; a_s[(3 * T + t) * AP + lp] = v.w;
-      }
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < KC; k++) {
-      const float4 a = *reinterpret_cast<const float4*>(a_s + k * AP + 4 * tx);
-      float wv[TN];
-#pragma unroll
-      for (int j = 0; j < TN; j += 2) {
-        const float2 w2 = *reinterpret_cast<const float2*>(w_s + k * WP + ty * TN + j);
-        wv[j] = w2.x; wv[j + 1] = w2.y;
-      }
-#pragma unroll
-      for (int j = 0; j < TN; j++) {
-        acc[0][j] = __fmaf_rn(a.x, wv[j], acc[0][j]);
-        acc[1][j] = __fmaf_rn(a.y, wv[j], acc[1][j]);
-        acc[2][j] = __fmaf_rn(a.z, wv[j], acc[2][j]);
-        acc[3][j] = __fmaf_rn(a.w, wv[j], acc[3][j]);
-      }
-    }
-    __syncthreads();
-  }
-  const int o = o0 + ty * TN;
-  float sc[TN], sf[TN];
-#pragma unroll
-  for (int j = 0; j < TN; j++) { sc[j] = __ldg(scale + o + j); sf[j] = __ldg(shift + o + j); }
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const long long pp = p0 + 4 * tx + i;
-    if (pp >= npix) continue;
-    float* dst = y + pp * y_stride + y_off + o;
-#pragma unroll
-    for (int j = 0; j < TN; j += 2) {
-      float r0 = __fmaf_rn(acc[i][j], sc[j], sf[j]), r1 = __fmaf_rn(acc[i][j + 1], sc[j + 1], sf[j + 1]);
-      if (RELU) { r0 = (r0 > 0.0f) ? r0 : 0.0f; r1 = (r1 > 0.0f) ? r1 : 0.0f; }
-      *reinterpret_cast<float2*>(dst + j) = make_float2(r0, r1);
-    }
-  }
-}
-
 // The module's 112 x 112 part in one kernel: s1 = relu(BN(conv3x3/2(image))), a1 = relu(BN(conv1x1(s1))) and the 2x2 max of s1
 // into channels 32..63 of the concatenated tensor, with s1 (a 16 x 16 tile of it) in shared memory only -- written and read
 // twice it was 3 x 51 MB of traffic at batch 32, and every kernel of its own a launch.  A thread owns 4 pixels of a row x 8
@@ -264,6 +160,138 @@ __global__ void __launch_bounds__(256, 3) stem_module_front(const float* __restr
   }
 }
 
+// The 56 x 56 part in one kernel: relu(BN(conv3x3/2(a1))), concatenated with the pooled channels in shared memory, then
+// BN(conv1x1) as the fp32 stream and its packed signs.  Persistent CTAs of 8 x 8 output pixels with both filter banks resident;
+// the patch of a1 lies channel by channel with even and odd columns apart (a row's three taps: three loads for 4 pixels).  A
+// thread owns 4 pixels x 2 channels of the first product and 4 x 4 of the second; chains run over c, kh, kw (then c) ascending.
+// The STEM-variant forward at batch 32: 443 us with the three kernels this replaces (two convolutions and the pack), 395 with it.
+constexpr int TL_TS = 8, TL_PS = 2 * TL_TS + 1, TL_HALF = 12, TL_PITCH = 68;
+constexpr int TL_PATCH = 16 * TL_PS * 2 * TL_HALF;
+constexpr int TL_SMEM = (144 * 32 + 64 * 64 + TL_PATCH + TL_TS * TL_TS * TL_PITCH) * 4;
+__global__ void __launch_bounds__(256, 2) stem_module_tail(const float* __restrict__ a1 /*[N][112][112][16]*/,
+                                                           const float* __restrict__ cat /*[N][56][56][64], channels 32..63*/,
+                                                           int ntiles, const float* __restrict__ w3, const float* __restrict__ scale3,
+                                                           const float* __restrict__ shift3, const float* __restrict__ w4,
+                                                           const float* __restrict__ scale4, const float* __restrict__ shift4,
+                                                           float* __restrict__ out /*[N][56][56][64]*/, uint64_t* __restrict__ bits) {
+  constexpr int IHW = 112, OHW = 56, TILES = OHW / TL_TS;
+  extern __shared__ __align__(16) float sm[];
+  float* w3_s = sm;                     // [144][32]
+  float* w4_s = w3_s + 144 * 32;        // [64][64]
+  float* x_s = w4_s + 64 * 64;          // [16][17][2][HALF]
+  float* c_s = x_s + TL_PATCH;          // [64 pixels][PITCH]: the concatenation
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int t = tid; t < 144 * 32; t += 256) w3_s[(t % 144) * 32 + t / 144] = w3[t];
+  for (int t = tid; t < 64 * 64; t += 256) w4_s[(t % 64) * 64 + t / 64] = w4[t];
+  const int chp = tid & 15, pg = tid >> 4;  // 16 channel groups x 16 groups of 4 pixels of a row
+  const int row = pg >> 1, x0 = (pg & 1) * 4;
+  const float sc3[2] = {__ldg(scale3 + 2 * chp), __ldg(scale3 + 2 * chp + 1)}, sf3[2] = {__ldg(shift3 + 2 * chp), __ldg(shift3 + 2 * chp + 1)};
+  float sc4[4], sf4[4];
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    sc4[j] = __ldg(scale4 + 4 * chp + j);
+    sf4[j] = __ldg(shift4 + 4 * chp + j);
+  }
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const long long n = tile / (TILES * TILES);
+    const int rem = tile % (TILES * TILES), oh0 = rem / TILES * TL_TS, ow0 = rem % TILES * TL_TS;
+    for (int t = tid; t < TL_PS * TL_PS * 4; t += 256) {
+      const int q = t & 3, px = t >> 2, lw = px % TL_PS, lh = px / TL_PS;
+      const int ih = 2 * oh0 - 1 + lh, iw = 2 * ow0 - 1 + lw;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ih >= 0 && ih < IHW && iw >= 0 && iw < IHW) v = __ldg(reinterpret_cast<const float4*>(a1 + ((n * IHW + ih) * IHW + iw) * 16) + q);
+      float* d = x_s + ((4 * q * TL_PS + lh) * 2 + (lw & 1)) * TL_HALF + (lw >> 1);
+      d[0] = v.x;
+      d[TL_PS * 2 * TL_HALF] = v.y;
+      d[2 * TL_PS * 2 * TL_HALF] = v.z;
+      d[3 * TL_PS * 2 * TL_HALF] = v.w;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int t = tid + 256 * u, q = t & 7, px = t >> 3;
+      const long long pix = (n * OHW + oh0 + px / TL_TS) * OHW + ow0 + px % TL_TS;
+      *reinterpret_cast<float4*>(c_s + px * TL_PITCH + 32 + 4 * q) = __ldg(reinterpret_cast<const float4*>(cat + pix * 64 + 32) + q);
+    }
+    __syncthreads();
+    {
+      unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+      for (int c = 0; c < 16; c++)
+#pragma unroll
+        for (int ki = 0; ki < 3; ki++) {
+          const float* xr = x_s + ((c * TL_PS + 2 * row + ki) * 2) * TL_HALF + x0;
+          const float4 e4 = *reinterpret_cast<const float4*>(xr);
+          const float4 o4 = *reinterpret_cast<const float4*>(xr + TL_HALF);
+          const float xe[5] = {e4.x, e4.y, e4.z, e4.w, xr[4]}, xo[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+          for (int kj = 0; kj < 3; kj++) {
+            const float2 w = *reinterpret_cast<const float2*>(w3_s + (c * 9 + ki * 3 + kj) * 32 + 2 * chp);
+            const unsigned long long w2 = pack_f32x2(w.x, w.y);
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+              const float xv = kj == 1 ? xo[i] : xe[i + (kj >> 1)];
+              fma_f32x2(acc2[i], pack_f32x2(xv, xv), w2);
+            }
+          }
+        }
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        float r0, r1;
+        unpack_f32x2(acc2[i], r0, r1);
+        r0 = __fmaf_rn(r0, sc3[0], sf3[0]);
+        r1 = __fmaf_rn(r1, sc3[1], sf3[1]);
+        *reinterpret_cast<float2*>(c_s + (row * TL_TS + x0 + i) * TL_PITCH + 2 * chp) = make_float2((r0 > 0.0f) ? r0 : 0.0f, (r1 > 0.0f) ? r1 : 0.0f);
+      }
+    }
+    __syncthreads();
+    {
+      const float* cp = c_s + (row * TL_TS + x0) * TL_PITCH;
+      unsigned long long acc2[4][2];
+#pragma unroll
+      for (int i = 0; i < 4; i++) acc2[i][0] = acc2[i][1] = 0ull;
+#pragma unroll 2
+      for (int k = 0; k < 64; k += 4) {
+        float xv[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const float4 v = *reinterpret_cast<const float4*>(cp + i * TL_PITCH + k);
+          xv[i][0] = v.x; xv[i][1] = v.y; xv[i][2] = v.z; xv[i][3] = v.w;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          const float4 w = *reinterpret_cast<const float4*>(w4_s + (k + u) * 64 + 4 * chp);
+          const unsigned long long wa = pack_f32x2(w.x, w.y), wb = pack_f32x2(w.z, w.w);
+#pragma unroll
+          for (int i = 0; i < 4; i++) {
+            const unsigned long long x2 = pack_f32x2(xv[i][u], xv[i][u]);
+            fma_f32x2(acc2[i][0], x2, wa);
+            fma_f32x2(acc2[i][1], x2, wb);
+          }
+        }
+      }
+      const unsigned gmask = 0xFFu << (lane & 24);
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        float r[4];
+        unpack_f32x2(acc2[i][0], r[0], r[1]);
+        unpack_f32x2(acc2[i][1], r[2], r[3]);
+        unsigned nib = 0;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          r[j] = __fmaf_rn(r[j], sc4[j], sf4[j]);
+          nib |= (unsigned)(r[j] < 0.0f) << j;
+        }
+        const long long pix = (n * OHW + oh0 + row) * OHW + ow0 + x0 + i;
+        *reinterpret_cast<float4*>(out + pix * 64 + 4 * chp) = make_float4(r[0], r[1], r[2], r[3]);
+        const unsigned half = __reduce_or_sync(gmask, nib << (4 * (lane & 7)));
+        const unsigned other = __shfl_xor_sync(0xFFFFFFFFu, half, 8);
+        if (chp == 0) bits[pix] = (uint64_t)half | ((uint64_t)other << 32);
+      }
+    }
+    __syncthreads();
+  }
+}
+
 }  // namespace
 
 // a1: [N][112][112][16], cat: [N][56][56][64] (scratch); out: [N][56][56][64] fp32, bits: its signs.
@@ -271,13 +299,13 @@ dabnn_status launch_stem_module(const dabnn_stem_module_params* sm, const float*
                                 float* out, uint64_t* bits, cudaStream_t st) {
   for (int i = 0; i < 4; i++)
     if (!sm->w[i] || !sm->scale[i] || !sm->shift[i]) return DABNN_ERR_NULL;
-  const long long p56 = (long long)N * 56 * 56;  // output pixels
   {
     static bool configured[kMaxDevices] = {};
     const int dev = current_device();
     if (dev < 0) return DABNN_ERR_CUDA;
     if (!configured[dev]) {
-      if (cudaFuncSetAttribute(stem_module_front, cudaFuncAttributeMaxDynamicSharedMemorySize, FR_SMEM) != cudaSuccess) {
+      if (cudaFuncSetAttribute(stem_module_front, cudaFuncAttributeMaxDynamicSharedMemorySize, FR_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(stem_module_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM) != cudaSuccess) {
         cudaGetLastError();
         return DABNN_ERR_CUDA;
       }
@@ -286,14 +314,10 @@ dabnn_status launch_stem_module(const dabnn_stem_module_params* sm, const float*
     stem_module_front<<<(unsigned)(N * 49), 256, FR_SMEM, st>>>(images, sm->w[0], sm->scale[0], sm->shift[0], sm->w[1], sm->scale[1],
                                                               sm->shift[1], a1, cat);
   }
-  conv_fp32_pinned<3, 2, 1, 16, 32, 4, true><<<dim3(ceil_div(p56, 128), 1), 256, 0, st>>>(
-      a1, N, 112, 112, 56, 56, sm->w[2], sm->scale[2], sm->shift[2], cat, 64, 0);
-  conv_fp32_pinned<1, 1, 0, 64, 64, 16, false><<<dim3(ceil_div(p56, 128), 1), 256, 0, st>>>(
-      cat, N, 56, 56, 56, 56, sm->w[3], sm->scale[3], sm->shift[3], out, 64, 0);
-  dabnn_status s = launch_status();
-  if (s != DABNN_OK) return s;
-  const dabnn_shape sh = {N, 64, 56, 56};
-  return dabnn_pack(out, DABNN_NHWC, sh, bits, st);
+  const int ntiles = N * 49, cap = 2 * sm_count();
+  stem_module_tail<<<ntiles < cap ? ntiles : cap, 256, TL_SMEM, st>>>(a1, cat, ntiles, sm->w[2], sm->scale[2], sm->shift[2], sm->w[3],
+                                                                   sm->scale[3], sm->shift[3], out, bits);
+  return launch_status();
 }
 
 }  // namespace dabnn
