@@ -148,6 +148,22 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   }
   return false;
 }
+// Waits for an asynchronous operation that this CTA has started (a bulk copy into its shared memory, its last MMAs) before the
+// CTA gives up what that operation still uses: bounded, but neither by the launch's limit nor by a failure elsewhere.  Returns
+// at once where the operation has completed, as it has in every launch whose waits did not run out.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  for (int tries = 0; tries < TC_WAIT_POLLS; tries++) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x400;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return;
+  }
+}
 // Address of the leader CTA's copy of a shared-memory object, in the cluster's shared window; arrive on it.
 __device__ __forceinline__ uint32_t leader_addr(uint32_t local) {
   uint32_t r;
@@ -291,6 +307,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 160);
   volatile int* s_fail = reinterpret_cast<volatile int*>(misc + 168);
   constexpr int B_RAW = 19, B_EXPANDED = 22;  // the packed weight rows have landed / have been expanded
+  constexpr int B_DRAIN = 23;  // (after a failed wait only) everything that the MMA thread has issued is done
   // [32 + 4 * e ..]: `res_full` of epilogue warp e's ring of residual chunks
   constexpr int B_RES_FULL = 32;
   float* s_scale = reinterpret_cast<float*>(misc + TC_SMEM_HDR);  // [nres][NT] this CTA's channels
@@ -323,6 +340,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       for (int i = 0; i < 3; i++) mbar_init(smem_u32(&bars[B_W_FULL + i]), (uint32_t)(rb_n + (i == 0 ? 4 : 0)) * PEERS);
       mbar_init(smem_u32(&bars[B_RAW]), 1);
       mbar_init(smem_u32(&bars[B_EXPANDED]), (uint32_t)(thirds ? 3 * rb_n : rb_n));
+      mbar_init(smem_u32(&bars[B_DRAIN]), 1);
       if (RES_TMA)
         for (int i = 0; i < 8 * TC_RING_MAX; i++) mbar_init(smem_u32(&bars[B_RES_FULL + i]), 1);  // the warp's issuing lane
       *s_fail = 0;
@@ -587,7 +605,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         commit(smem_u32(&bars[B_A_FREE + ab]));  // the tile's rows have been read: the A buffer may be refilled
         if (++ab == (uint32_t)g.abufs) { ab = 0; a_phase ^= 1u; }
       }
+      if (*s_fail != 0) {  // MMAs of earlier tiles may still read shared memory and write accumulators
+        const uint32_t bar = smem_u32(&bars[B_DRAIN]);
+        if (PAIR) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+        else asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+        mbar_drain(smem_u32(&bars[B_DRAIN]), 0);
+      }
     }
+    // the bulk copies that this thread has requested: after a failed wait they may still be on their way
+    if (lane == 0) mbar_drain(smem_u32(&bars[B_RAW]), 0);
+    __syncwarp();
   } else if (warp >= 4 && warp < 8) {
     // ================= producer warps: packed bits -> e2m1 rows ===================================================
     const int ptid = tid - 128;
@@ -1070,7 +1097,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     }
     // (only after a wait ran out:) chunks still on their way must land before the CTA gives up its shared memory
     while (tma_res && in_flight > 0) {
-      __all_sync(0xFFFFFFFFu, mbar_wait(rbar0 + 8u * slot_u, phase_u, s_fail, g.wait_polls));
+      mbar_drain(rbar0 + 8u * slot_u, phase_u);
       in_flight--;
       if (++slot_u == (uint32_t)g.res_ring) { slot_u = 0; phase_u ^= 1u; }
     }

@@ -299,6 +299,13 @@ def test_a_wait_that_runs_out_sets_the_flag_and_leaves_the_device_usable(B, orac
             got = B.tc_bconv2d(a, wt, (1, 1), (pad, pad), -1, B.NHWC).cpu().numpy()
             assert np.array_equal(got, want)
         assert B.last_device_flag() == 0
+        # limits shorter than the CTA's own weight copy takes: every role gives up while the copy may still be on its way, and
+        # the kernel must not hand its shared memory on before that copy has landed
+        for polls in (1, 2, 3):
+            for _ in range(8):
+                B.tc_wait_expiry_selftest(a, wt, (1, 1), (pad, pad), -1, wait_polls=polls)
+                assert np.array_equal(B.tc_bconv2d(a, wt, (1, 1), (pad, pad), -1, B.NHWC).cpu().numpy(), want)
+            assert B.stream_status() == B.ERR_TIMEOUT
     with pytest.raises(B.DabnnError):
         B.tc_wait_expiry_selftest(a, wt, (1, 1), (pad, pad), -1, wait_polls=1 << 20)  # limit beyond a few milliseconds: refused
 
