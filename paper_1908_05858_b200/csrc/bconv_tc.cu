@@ -1400,13 +1400,16 @@ void tc_plan(TcArgs& g, int O, int C, int taps) {
   // some 400.  1x1, 128 -> 512 channels at 28x28, batch 16: 21.6 -> 15.1 us against "as many as leave every unit a tile".
   const long long acc_cyc = (long long)taps * g.Cw * 70 > 2000 ? (long long)taps * g.Cw * 70 : 2000;
   const long long exp_cyc = 600 + 200LL * g.Cw;
+  // Every group needs a unit of its own (a pair of CTAs may not find a place on every pair of SMs, hence the margin); with more
+  // groups than that at every count, the largest count gives the launch its best chance.
+  const long long most = pair ? units2 - 8 : units1;
   long long best = -1;
-  int best_n = 1;
+  int best_n = (int)nres;
   for (int n = (int)nres; n >= 1; n--) {
     const long long groups = (g.n_ntiles + n - 1) / n;
+    if (groups > most) break;
     const long long per = (pair ? units2 : units1) / groups;  // units that share a group's tiles
-    if (per <= 0 && n > 1) continue;
-    const long long rounds = per > 0 ? (m_units + per - 1) / per : m_units;
+    const long long rounds = (m_units + per - 1) / per;
     const long long cost = rounds * ((n * acc_cyc > exp_cyc ? n * acc_cyc : exp_cyc) + 400) + n * wr * Kb / 256;
     if (best < 0 || cost < best) {
       best = cost;

@@ -238,6 +238,19 @@ def test_tc_sign_epilogue_is_exact_for_awkward_bn_vectors(B, oracle_mod, C, k, p
     assert B.tc_error_flag() == 0
 
 
+@pytest.mark.parametrize("N", [148 * 128 + 1, 25600, 4 * 148 * 128])
+def test_tc_bgemm_with_more_channel_tiles_than_ctas(B, oracle_mod, N):
+    """More tiles of 128 output channels than there are CTAs: several of them have to be resident in each (up to four)."""
+    M, K = 70, 512
+    rng = np.random.default_rng(N)
+    A = B.pack(dev(rng.standard_normal((M, K, 1, 1)).astype(np.float32))).reshape(M, -1)
+    Bp = torch.from_numpy(rng.integers(-2**63, 2**63, (N, 1, 1, K // 64), dtype=np.int64)).cuda()
+    got = B.tc_bgemm(A, B.TcWeights(Bp, K), K).cpu().numpy()
+    counts = oracle_mod.bgemm_xnor(u64(A), u64(Bp).reshape(N, -1), K)
+    assert np.array_equal(got, 2 * counts - K)
+    assert B.tc_error_flag() == 0
+
+
 @pytest.mark.parametrize("cap", [1, 10, 74])
 def test_tc_results_do_not_depend_on_the_cta_cap(B, oracle_mod, cap):
     o = oracle_mod
