@@ -430,15 +430,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     }
   }
   // The start-up barrier: barriers initialised (in both CTAs of a pair, before either signals the other's), per-channel
-  // constants written and the tensor-memory address published.
-  auto prologue_sync = [&]() {
+  // constants written and the tensor-memory address published.  The producers only arrive here: they wait with their first
+  // requests for activation bits out (see `run`), so that neither the coordinates of their rows hold up the other roles nor the
+  // start-up holds up the requests.
+  const bool is_producer = warp >= 4 && warp < 8;
+  __syncwarp();
+  if (PAIR) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (PAIR) cluster_sync_all();
-    else __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  } else if (is_producer) {
+    asm volatile("barrier.cta.arrive 1, %0;" ::"n"(TC_THREADS) : "memory");  // what the others wait for
+  } else {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("barrier.cta.arrive 2, %0;" ::"n"(TC_THREADS) : "memory");  // what the producers wait for
+  }
+  auto prologue_wait = [&]() {
+    if (PAIR) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else if (is_producer) asm volatile("barrier.cta.sync 2, %0;" ::"n"(TC_THREADS) : "memory");
+    else asm volatile("barrier.cta.sync 1, %0;" ::"n"(TC_THREADS) : "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   };
-  prologue_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  if (!is_producer) prologue_wait();
+  const uint32_t tmem_base = is_producer ? 0u : *tmem_slot;  // (the producers never touch tensor memory)
   // barriers that both CTAs of a pair signal live in the leader
   const uint32_t bar_tmem_free0 = PAIR ? leader_addr(smem_u32(&bars[B_TMEM_FREE])) : smem_u32(&bars[B_TMEM_FREE]);
   const uint32_t bar_a_full0 = PAIR ? leader_addr(smem_u32(&bars[B_A_FULL])) : smem_u32(&bars[B_A_FULL]);
@@ -697,24 +710,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       }
     };
 
-    {
-      // every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout (each warp: its quarter of the rows).
-      // Here, before this role holds a tile's words in registers: after the first tile, or in the epilogue warps, it costs spills.
-      const uint32_t one = 0x7F7F7F7Fu;
-#pragma unroll 1
-      for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
-        const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c;
-        asm volatile(
-            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
-            "r"(one)
-            : "memory");
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) arrive(bar_w_full);
-    }
-    chain_wait();
     int it = 0;
     // Per tile: wait until the A buffer is free, expand the rows held in `cur`, hand them over, move the next tile's
     // bits (requested one tile ago, so they have landed) from `nxt` into `cur`, and request the tile after that into
@@ -725,8 +720,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       constexpr bool TWO_SETS = SPT <= 2;
       SlotRegs cur, nxt;
       long long mt = mt_first;
+      // The first requests are out before the start-up barrier is waited for: of a 1x1, stride-2 launch over 512 channels 0.9 of
+      // 9.9 us.  (A chained launch has its start-up behind it when the previous kernel ends.)
+      chain_wait();
       prefetch(cur, cwc);  // (rows of a tile beyond the last one are beyond the batch: nothing is read for them)
       if (TWO_SETS) prefetch(nxt, cwc);
+      prologue_wait();
       uint32_t ab = 0, use_phase = 0;  // A buffer of this tile and the parity of the number of times it has been filled
       bool stop = false;
 #pragma unroll 1
@@ -762,7 +761,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     else if (g.Cw == 1) run(IntC<1>{});
     else if (g.Cw == 2) run(IntC<2>{});
     else if (g.Cw <= 4) run(IntC<4>{});
-    else if constexpr (PCW > 4) run(IntC<8>{});  // (where PCW is 4 the host launches this instance for C <= 256 only)
+    else if constexpr (PCW > 4) run(IntC<8>{});
+    else prologue_wait();  // (not reached: where PCW is 4 the host launches this instance for C <= 256 only)
   } else {
     // ================= epilogue warps: the resident weights, then TMEM accumulator -> output =====================
     const bool has_epi = warp < 4 || g.epi2;
@@ -825,6 +825,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     // 3x3, C = 256 CTA are in place after 7.5 k cycles instead of 10 k.
     {
       constexpr int BATCH = 3;
+      if (warp >= 8) {
+        // while the packed rows are on their way: every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their
+        // layout (each warp: its quarter of the rows)
+        const uint32_t one = 0x7F7F7F7Fu;
+#pragma unroll 1
+        for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
+          const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c;
+          asm volatile(
+              "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+              "r"(one)
+              : "memory");
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) arrive(bar_w_full);
+      }
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
       const int K64 = g.kh * g.kw * g.Cw;
       const uint64_t* raw = reinterpret_cast<const uint64_t*>(a_s + g.raw_off);
