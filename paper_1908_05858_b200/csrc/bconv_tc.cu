@@ -207,15 +207,12 @@ __device__ __forceinline__ uint4 expand32(uint32_t w) {
   return make_uint4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// Expanded nibbles of the channels whose bit in `valid` is 0 become e2m1 0.0: they contribute nothing.  The validity bits go
-// through the same expansion (and so the same channel order): 0xA marks a live nibble.
-__device__ __forceinline__ uint4 mask_channels(uint4 bytes, uint32_t valid) {
+// A mask that makes the expanded nibbles of the channels whose bit in `valid` is 0 e2m1 0.0: they contribute nothing.  The
+// validity bits go through the same expansion (and so the same channel order): 0xA marks a live nibble.
+__device__ __forceinline__ uint4 channel_mask(uint32_t valid) {
   const uint4 v = expand32(valid);
-  bytes.x &= ((v.x >> 3) & 0x11111111u) * 0xFu;
-  bytes.y &= ((v.y >> 3) & 0x11111111u) * 0xFu;
-  bytes.z &= ((v.z >> 3) & 0x11111111u) * 0xFu;
-  bytes.w &= ((v.w >> 3) & 0x11111111u) * 0xFu;
-  return bytes;
+  return make_uint4(((v.x >> 3) & 0x11111111u) * 0xFu, ((v.y >> 3) & 0x11111111u) * 0xFu, ((v.z >> 3) & 0x11111111u) * 0xFu,
+                    ((v.w >> 3) & 0x11111111u) * 0xFu);
 }
 
 // 256-bit global store / load (32-byte aligned): a lane writes a whole 32-byte sector of its output row at once.
@@ -844,6 +841,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       }
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
       const int K64 = g.kh * g.kw * g.Cw;
+      // Channel tails: where in its row of Cw words a lane's word lies goes along with it (4 words a step, no division), and the
+      // mask of the last word is made once.  3x3, 168 -> 82 channels, one 56x58 image, stride 2, sign words: 10.5 -> 10.1 us
+      const bool tail = g.w_tail != ~0ull;
+      const int cw_first = (lane >> 3) % g.Cw, cw_step = 4 % g.Cw;
+      const uint4 tail_lo = channel_mask((uint32_t)g.w_tail), tail_hi = channel_mask((uint32_t)(g.w_tail >> 32));
       const uint64_t* raw = reinterpret_cast<const uint64_t*>(a_s + g.raw_off);
 #pragma unroll 1
       for (int item = warp < 4 ? warp : warp - 4; item < (thirds ? 3 * rb_n : rb_n); item += 8) {
@@ -853,6 +855,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         const bool exists = (ng * g.nres + r) * NT + (int)rank * WR + n < g.O;  // (beyond O: zero weights)
         const uint64_t* src = raw + row * K64;
         uint8_t* dst = w_s + (size_t)(2 * r * K64 * WR + n) * 16;
+        int cw = cw_first;  // (k_lo is a multiple of Cw)
 #pragma unroll 1
         for (int k = k_lo + (lane >> 3); k < k_hi; k += 4 * BATCH) {
           uint64_t word[BATCH];
@@ -862,9 +865,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
           for (int u = 0; u < BATCH; u++) {
             if (k + 4 * u >= k_hi) break;
             uint4 lo = expand32((uint32_t)word[u]), hi = expand32((uint32_t)(word[u] >> 32));
-            if (g.w_tail != ~0ull && (k + 4 * u) % g.Cw == g.Cw - 1) {  // (channel tails only)
-              lo = mask_channels(lo, (uint32_t)g.w_tail);
-              hi = mask_channels(hi, (uint32_t)(g.w_tail >> 32));
+            if (tail) {
+              if (cw == g.Cw - 1) {
+                lo.x &= tail_lo.x; lo.y &= tail_lo.y; lo.z &= tail_lo.z; lo.w &= tail_lo.w;
+                hi.x &= tail_hi.x; hi.y &= tail_hi.y; hi.z &= tail_hi.z; hi.w &= tail_hi.w;
+              }
+              cw += cw_step;
+              if (cw >= g.Cw) cw -= g.Cw;
             }
             if (!exists) lo = hi = make_uint4(0, 0, 0, 0);
             *reinterpret_cast<uint4*>(dst + (size_t)(2 * (k + 4 * u)) * WR * 16) = lo;
