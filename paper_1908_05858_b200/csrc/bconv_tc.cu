@@ -1379,8 +1379,12 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   return DABNN_ERR_UNSUPPORTED;
 }
 
+void tc_plan(TcArgs& g, int epi);
+
 template <int EPI>
 dabnn_status tc_dispatch(TcArgs& g, cudaStream_t st) {
+  tc_plan(g, EPI);
+  if (g.ntile == 0) return DABNN_ERR_UNSUPPORTED;
   // A second group of epilogue warps (measured): it pays for the residual epilogue, which moves two fp32 rows per
   // output row; elsewhere the extra warps only add contention.
   // (environment DABNN_TC_EPI2 = 0 / 1 overrides, for measurements)
@@ -1393,9 +1397,18 @@ dabnn_status tc_dispatch(TcArgs& g, cudaStream_t st) {
   return g.pair ? tc_dispatch_mode<EPI, true>(g, st) : tc_dispatch_mode<EPI, false>(g, st);
 }
 
+// Output rows leave as whole 32-byte pieces (or, in NCHW order, as whole lines of consecutive pixels), not as 4-byte stores
+// scattered over them.
+bool tc_wide_rows(const TcArgs& g, int epi) {
+  if (epi == EPI_BNPACK || (epi == EPI_I32 && g.out_nchw)) return true;
+  if (g.O % 8 != 0) return false;
+  return epi == EPI_I32 ? aligned(g.out, 32) : aligned(g.residual, 32) && aligned(g.y_out, 32);
+}
+
 // Launch form for a problem: CTA pairs when there are enough tiles to fill the chip with pairs, and as many channel
 // tiles resident per CTA (pair) as fit while every CTA (pair) still gets work.
-void tc_plan(TcArgs& g, int O, int C, int taps) {
+void tc_plan(TcArgs& g, int epi) {
+  const int O = g.O, C = g.C, taps = g.kh * g.kw;
   const long long Kb = (long long)tc_cpad(C) / 2 * taps;
   const int mode = tc_mode();
   const int units1 = sm_count(), units2 = sm_count() / 2;
@@ -1418,12 +1431,17 @@ void tc_plan(TcArgs& g, int O, int C, int taps) {
   const long long m_units = pair ? (g.m_tiles + 1) / 2 : g.m_tiles;
   if (g.kgroups > 1) nres = 1;  // (the groups of a tile add up in one accumulator)
   // How many of them: the units of a launch are dealt to groups of channel tiles first, so the busiest unit does
-  // ceil(m_units / (units / groups)) tiles of nres accumulators each.  Few resident tiles deal more evenly, many expand each
-  // activation tile fewer times; per accumulator the MMAs or the epilogue set the pace (cycles measured: 70 per MMA of 128
-  // columns, about 2000 for the epilogue), per tile the expansion does (600 + 200 per word), and a tile's hand-over costs
-  // some 400.  1x1, 128 -> 512 channels at 28x28, batch 16: 21.6 -> 15.1 us against "as many as leave every unit a tile".
-  const long long acc_cyc = (long long)taps * g.Cw * 70 > 2000 ? (long long)taps * g.Cw * 70 : 2000;
-  const long long exp_cyc = 600 + 200LL * g.Cw;
+  // ceil(m_units / (units / groups)) tiles of nres accumulators each.  Few resident tiles deal more evenly and have fewer weights
+  // to expand first, many expand each activation tile fewer times.  In cycles, fitted to 435 launches timed with every count
+  // (16 to 512 channels, 1x1 and 3x3, strides 1 and 2, O 17 to 2048): per tile the slowest of the MMAs (70 each), the epilogue
+  // (per 128 channels that exist: int32 2000, sign words 1000, residual 4000; by 4-byte stores 16000 and 40000) and the expansion
+  // (300 + 150 per word and row of a producer thread); 300 to hand a tile over (100 beside 4-byte stores); 40 bytes of expanded
+  // weights a cycle.  Its choice takes 0.3 % longer than the best count on the mean and 15 % at most; a rule without the output
+  // form and the cost of the weights 1.9 % and 37 %, "as many as leave every unit a tile" 4.8 % and 85 %.
+  const bool wide = tc_wide_rows(g, epi);
+  const long long epi_cyc = epi == EPI_I32 ? (wide ? 2000 : 16000) : epi == EPI_BNPACK ? 1000 : (wide ? 4000 : 40000);
+  const long long mma_cyc = 70LL * taps * g.Cw, exp_cyc = 300 + 150LL * g.Cw * ((g.slots + 127) / 128), hand_cyc = wide ? 300 : 100;
+  const long long o_cols = epi == EPI_BNPACK ? (O + 63) / 64 * 64 : O;
   // Every group needs a unit of its own (a pair of CTAs may not find a place on every pair of SMs, hence the margin); with more
   // groups than that at every count, the largest count gives the launch its best chance.
   const long long most = pair ? units2 - 8 : units1;
@@ -1434,7 +1452,11 @@ void tc_plan(TcArgs& g, int O, int C, int taps) {
     if (groups > most) break;
     const long long per = (pair ? units2 : units1) / groups;  // units that share a group's tiles
     const long long rounds = (m_units + per - 1) / per;
-    const long long cost = rounds * ((n * acc_cyc > exp_cyc ? n * acc_cyc : exp_cyc) + 400) + n * wr * Kb / 256;
+    const long long live = (long long)n * g.ntile < o_cols ? (long long)n * g.ntile : o_cols;
+    long long tile = epi_cyc * live / 128;
+    if (tile < n * mma_cyc) tile = n * mma_cyc;
+    if (tile < exp_cyc) tile = exp_cyc;
+    const long long cost = rounds * (tile + hand_cyc) + n * wr * Kb / 40;
     if (best < 0 || cost < best) {
       best = cost;
       best_n = n;
@@ -1483,8 +1505,6 @@ dabnn_status tc_fill(TcArgs& g, const uint64_t* a, dabnn_shape in, const void* w
   // words per row that a producer thread holds: 8 (4 where it holds five rows, stride 2); more channels go in groups
   g.gw = g.slots <= 256 ? TC_MAX_CW : 4;
   g.kgroups = (g.Cw + g.gw - 1) / g.gw;
-  tc_plan(g, O, in.C, cv.kh * cv.kw);
-  if (g.ntile == 0) return DABNN_ERR_UNSUPPORTED;
   if ((long long)in.N * OH * OW >= (1LL << 31) || (long long)in.N * OH * OW * O > (1LL << 40)) return DABNN_ERR_UNSUPPORTED;
   g.pad_neg = cv.pad_value < 0;
   g.out = nullptr; g.out_nchw = 0; g.scale = g.shift = g.residual = nullptr; g.y_out = nullptr;
