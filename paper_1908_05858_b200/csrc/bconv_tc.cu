@@ -427,28 +427,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     }
   }
   // The start-up barrier: barriers initialised (in both CTAs of a pair, before either signals the other's), per-channel
-  // constants written and the tensor-memory address published.  The producers only arrive here: they wait with their first
-  // requests for activation bits out (see `run`), so that neither the coordinates of their rows hold up the other roles nor the
-  // start-up holds up the requests.
+  // constants written and the tensor-memory address published.  In the instances for any channel count the producers only arrive
+  // here: they wait with their first requests for activation bits out (see `run`), so that neither the coordinates of their rows
+  // hold up the other roles nor the start-up holds up the requests.  (Of a 1x1, stride-2 launch over 512 channels that is 0.9 of 9.9
+  // us, and their loops come out faster: 3x3, 1024 -> 1024, batch 64 at 14x14 244 -> 219.  The loops of the instances for one count
+  // come out slower by 1 to 5 % that way: 3x3, 512 -> 512, batch 15 at 42x42, 40.0 us as here, 42.3 otherwise.)
+  constexpr bool EARLY = CWX == 0;
   const bool is_producer = warp >= 4 && warp < 8;
-  __syncwarp();
-  if (PAIR) {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  } else if (is_producer) {
-    asm volatile("barrier.cta.arrive 1, %0;" ::"n"(TC_THREADS) : "memory");  // what the others wait for
-  } else {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    asm volatile("barrier.cta.arrive 2, %0;" ::"n"(TC_THREADS) : "memory");  // what the producers wait for
-  }
   auto prologue_wait = [&]() {
     if (PAIR) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     else if (is_producer) asm volatile("barrier.cta.sync 2, %0;" ::"n"(TC_THREADS) : "memory");
     else asm volatile("barrier.cta.sync 1, %0;" ::"n"(TC_THREADS) : "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   };
-  if (!is_producer) prologue_wait();
-  const uint32_t tmem_base = is_producer ? 0u : *tmem_slot;  // (the producers never touch tensor memory)
+  if constexpr (EARLY) {
+    __syncwarp();
+    if (PAIR) {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    } else if (is_producer) {
+      asm volatile("barrier.cta.arrive 1, %0;" ::"n"(TC_THREADS) : "memory");  // what the others wait for
+    } else {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      asm volatile("barrier.cta.arrive 2, %0;" ::"n"(TC_THREADS) : "memory");  // what the producers wait for
+    }
+    if (!is_producer) prologue_wait();
+  } else {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (PAIR) cluster_sync_all();
+    else __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  const uint32_t tmem_base = EARLY && is_producer ? 0u : *tmem_slot;  // (early producers never touch tensor memory)
   // barriers that both CTAs of a pair signal live in the leader
   const uint32_t bar_tmem_free0 = PAIR ? leader_addr(smem_u32(&bars[B_TMEM_FREE])) : smem_u32(&bars[B_TMEM_FREE]);
   const uint32_t bar_a_full0 = PAIR ? leader_addr(smem_u32(&bars[B_A_FULL])) : smem_u32(&bars[B_A_FULL]);
@@ -456,6 +466,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   auto arrive = [&](uint32_t bar) {
     if (PAIR) mbar_arrive_cluster(bar);
     else mbar_arrive(bar);
+  };
+  // Every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their layout (each of four warps: its quarter of the rows).
+  auto unit_scales = [&]() {
+    const uint32_t one = 0x7F7F7F7Fu;
+#pragma unroll 1
+    for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
+      const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c;
+      asm volatile(
+          "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+          "r"(one)
+          : "memory");
+    }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) arrive(bar_w_full);
   };
   // (chained launches: nothing above reads or writes what the previous kernel of the stream produces or still reads; a warp
   // waits for that kernel where it first touches the activation bits, the residual or an output.  A no-op in an ordinary launch.)
@@ -707,6 +733,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       }
     };
 
+    if constexpr (!EARLY) {
+      unit_scales();  // (here, before this role holds a tile's words in registers: after the first tile it costs spills)
+      chain_wait();
+    }
     int it = 0;
     // Per tile: wait until the A buffer is free, expand the rows held in `cur`, hand them over, move the next tile's
     // bits (requested one tile ago, so they have landed) from `nxt` into `cur`, and request the tile after that into
@@ -717,12 +747,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       constexpr bool TWO_SETS = SPT <= 2;
       SlotRegs cur, nxt;
       long long mt = mt_first;
-      // The first requests are out before the start-up barrier is waited for: of a 1x1, stride-2 launch over 512 channels 0.9 of
-      // 9.9 us.  (A chained launch has its start-up behind it when the previous kernel ends.)
-      chain_wait();
+      if constexpr (EARLY) chain_wait();  // (a chained launch has its start-up behind it when the previous kernel ends)
       prefetch(cur, cwc);  // (rows of a tile beyond the last one are beyond the batch: nothing is read for them)
       if (TWO_SETS) prefetch(nxt, cwc);
-      prologue_wait();
+      if constexpr (EARLY) prologue_wait();
       uint32_t ab = 0, use_phase = 0;  // A buffer of this tile and the parity of the number of times it has been filled
       bool stop = false;
 #pragma unroll 1
@@ -822,23 +850,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     // 3x3, C = 256 CTA are in place after 7.5 k cycles instead of 10 k.
     {
       constexpr int BATCH = 3;
-      if (warp >= 8) {
-        // while the packed rows are on their way: every byte of the scale-factor columns is ue8m0 127 = 1.0, whatever their
-        // layout (each warp: its quarter of the rows)
-        const uint32_t one = 0x7F7F7F7Fu;
-#pragma unroll 1
-        for (int c = TC_SF_COL; c < TC_TMEM_COLS; c += 16) {
-          const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c;
-          asm volatile(
-              "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
-              "r"(one)
-              : "memory");
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) arrive(bar_w_full);
-      }
+      if (EARLY && warp >= 8) unit_scales();  // (while the packed rows are on their way)
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&bars[B_RAW]), 0, s_fail, g.wait_polls))) *s_fail = 1;
       const int K64 = g.kh * g.kw * g.Cw;
       // Channel tails: where in its row of Cw words a lane's word lies goes along with it (4 words a step, no division), and the
