@@ -798,7 +798,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     const int c_first = warp >= 8 && !ALTERNATE ? 32 : 0;
     const int c_step = g.epi2 && !ALTERNATE ? 64 : 32;
     uint32_t round = warp >= 8 ? 1u : 0u;  // (ALTERNATE) even: this group's accumulator
-    const bool wide_bits = ALTERNATE && g.epi2 && (g.Ow32 & 3) == 0 && (reinterpret_cast<uintptr_t>(g.out_packed32) & 15) == 0;
+    // (without a second group the assembly costs single CTAs up to 3 %, 3x3, 64 -> 256, batch 192 at 55x55 81.6 us as here, 84.0 with it;
+    // pairs gain from it: 3x3, 512 -> 512, batch 15 at 42x42 40.5 us with it, 42.2 without)
+    const bool wide_bits = ALTERNATE && (PAIR || g.epi2) && (g.Ow32 & 3) == 0 && (reinterpret_cast<uintptr_t>(g.out_packed32) & 15) == 0;
     const uint64_t pol_stream = EPI == EPI_I32 ? evict_first_policy() : 0ull;  // (made once, not per store)
     // The residual as bulk tensor copies (g.res_ring > 0): every epilogue warp owns a ring of 4 KB chunks (32 rows x 32
     // channels) and its lane 0 requests the chunks in the order the warp will use them, `res_ring` chunks ahead -- across
