@@ -255,6 +255,7 @@ dabnn_status dabnn_binary_layer_host(const float* x_host, dabnn_shape in, const 
  *                             The buffer's content belongs to the library version that wrote it (at present the packed
  *                             words: each CTA expands its own rows on chip)
  *   dabnn_tc_bconv2d*         as dabnn_bconv2d*, with w_tc in place of w_packed
+ *   dabnn_tc_launches         launches of this engine that this process has made so far, whichever call made them
  *   dabnn_tc_error_flag       synchronises nothing itself; copies the current device's error flag (1 if a bounded wait
  *                             inside a kernel ran out since the flag was last cleared, else 0; -1 if it cannot be read)
  *                             and leaves it set.  Call after synchronising the stream.
@@ -281,6 +282,7 @@ dabnn_status dabnn_tc_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_s
 /* Eq. 1 (BGEMM) on the tensor-core engine: dabnn_bgemm with B prepared once by
  * dabnn_tc_prepare_weights(B, N, Kbits, 1, 1, b_tc) (dabnn_tc_weights_bytes(N, Kbits, 1, 1) bytes; Kbits <= 512).  Same integers. */
 dabnn_status dabnn_tc_bgemm(const uint64_t* A, int M, const void* b_tc, int N, int Kbits, int32_t* C, void* stream);
+unsigned long long dabnn_tc_launches(void);
 int dabnn_tc_error_flag(void);
 int dabnn_last_device_flag(void* stream);
 dabnn_status dabnn_stream_status(void* stream);

@@ -29,7 +29,7 @@ EXPORTS = (
     "dabnn_tc_set_max_ctas", "dabnn_tc_weights_bytes", "dabnn_tc_prepare_weights", "dabnn_tc_bconv2d", "dabnn_tc_bconv2d_bn_sign_pack",
     "dabnn_tc_bconv2d_bn_add_sign_pack", "dabnn_tc_error_flag", "dabnn_last_device_flag", "dabnn_stream_status",
     "dabnn_tc_wait_expiry_selftest", "dabnn_packed_words", "dabnn_pack_as", "dabnn_bconv2d_from",
-    "dabnn_bireal18_forward_stem_module", "dabnn_tc_bgemm",
+    "dabnn_bireal18_forward_stem_module", "dabnn_tc_bgemm", "dabnn_tc_launches",
 )
 
 PACKED_NHWC = 0
@@ -114,6 +114,8 @@ def lib() -> ctypes.CDLL:
         for name in ("dabnn_tc_prepare_weights", "dabnn_tc_bconv2d", "dabnn_tc_bconv2d_bn_sign_pack",
                      "dabnn_tc_bconv2d_bn_add_sign_pack", "dabnn_tc_error_flag"):
             getattr(L, name).restype = ci
+        L.dabnn_tc_launches.restype = ctypes.c_ulonglong
+        L.dabnn_tc_launches.argtypes = []
         L.dabnn_set_conv_tile.restype = ci
         L.dabnn_set_conv_tile.argtypes = [ci]
         L.dabnn_bireal18_forward_stem_module.restype = ci
@@ -564,6 +566,11 @@ def tc_bgemm(A: torch.Tensor, Bt: "TcWeights", Kbits: int) -> torch.Tensor:
 def tc_set_max_ctas(max_ctas: int) -> int:
     """dabnn_tc_set_max_ctas: cap the CTAs of a tensor-engine launch (0 = all SMs); returns the previous setting."""
     return int(lib().dabnn_tc_set_max_ctas(int(max_ctas)))
+
+
+def tc_launches() -> int:
+    """dabnn_tc_launches: launches of the tensor-core engine that this process has made so far."""
+    return int(lib().dabnn_tc_launches())
 
 
 def tc_error_flag() -> int:

@@ -87,22 +87,25 @@ dabnn_status launch_tile(const BConvArgs& g, bool csa, cudaStream_t st) {
                : launch_one<BP, BO, TP, TO, MINB, EPI, false, false, STAGES>(g, st);
 }
 
+long long tile_ctas(long long M, int ochan, int bp, int bo) { return ((M + bp - 1) / bp) * ((ochan + bo - 1) / bo); }
+
+// Measured on B200 (batch 64 to 256, the ResNet-18 stage shapes and the 1x1 512 -> 2048 layer): 32 outputs per thread
+// (128 x 64, two CTAs = 16 warps per SM) where that still gives four waves of CTAs, else 16 outputs per thread (64 x 64);
+// the 8 x 8 register tile of 128 x 128 spills at 255 registers, leaves two warps per scheduler and is slower everywhere.
+int choose_tile(long long M, int ochan, long long K64, int sms) {
+  if (tile_ctas(M, ochan, 128, 64) >= 4LL * sms) return 2;
+  if (tile_ctas(M, ochan, 64, 64) >= 4LL * sms) return 3;
+  if (tile_ctas(M, ochan, 32, 32) >= sms || K64 > 5 * KC64) return 4;
+  return 5;  // less than one wave of the smallest tile: latency is all that counts
+}
+
 template <int EPI>
 dabnn_status launch_epi(const BConvArgs& g, cudaStream_t st) {
   const bool csa = g_conv_variant != 1;
   const int sms = sm_count();
   const int ochan = (EPI == EPI_I32) ? g.O : g.Ow32 * 32;
-  auto ctas = [&](int bp, int bo) { return ((g.M + bp - 1) / bp) * ((ochan + bo - 1) / bo); };
-  int tile = g_conv_tile;
-  if (tile == 0) {
-    // Measured on B200 (batch 64 to 256, the ResNet-18 stage shapes and the 1x1 512 -> 2048 layer): 32 outputs per thread
-    // (128 x 64, two CTAs = 16 warps per SM) where that still gives four waves of CTAs, else 16 outputs per thread (64 x 64);
-    // the 8 x 8 register tile of 128 x 128 spills at 255 registers, leaves two warps per scheduler and is slower everywhere.
-    if (ctas(128, 64) >= 4LL * sms) tile = 2;
-    else if (ctas(64, 64) >= 4LL * sms) tile = 3;
-    else if (ctas(32, 32) >= sms || g.K64 > 5 * KC64) tile = 4;
-    else tile = 5;  // less than one wave of the smallest tile: latency is all that counts
-  }
+  auto ctas = [&](int bp, int bo) { return tile_ctas(g.M, ochan, bp, bo); };
+  const int tile = g_conv_tile != 0 ? g_conv_tile : choose_tile(g.M, ochan, g.K64, sms);
   if constexpr (EPI != EPI_BIREAL) {
     // short-K pointwise layers with at least four waves of four-tile CTAs (DABNN_CONV_POINTWISE=0 in the environment, read
     // once, keeps the one-tile form, for measurements)
@@ -164,15 +167,40 @@ dabnn_status fill_args(BConvArgs& g, const uint64_t* a, dabnn_shape in, const ui
   return DABNN_OK;
 }
 
-// Packed-weight calls that run on the tensor-core engine (same integers, see tc_bits_worthwhile), unless a measurement
-// run has fixed the loop or the tile, or the call belongs to a chained forward whose caller gave no expanded weights.
-bool tensor_route(dabnn_shape in, const uint64_t* w, int O, dabnn_conv cv, int epi) {
+// Packed-weight calls go to the tensor-core engine (same integers) where that is estimated to be faster, unless a measurement
+// run has fixed the loop or the tile.
+bool tensor_route(const uint64_t* w) {
   if (!aligned(w, 16)) return false;  // (its weight rows are fetched with bulk copies)
-  if (g_conv_variant != 0 || g_conv_tile != 0 || g_chain_launch) return false;
-  return tc_bits_worthwhile(in, O, cv, epi);
+  return g_conv_variant == 0 && g_conv_tile == 0;
 }
 
 }  // namespace
+
+// Fitted (least squares of the relative error; 90 % of the launches within -12 and +12 %) to 3304 launches, those that the tensor-core
+// engine's estimate was fitted to and as many others.  What the two estimates choose together takes 0.5 % longer on the mean
+// than the better engine (0.3 % over 1x1 and 3x3 filters), and 2 % of the launches lose more than 5 %; an estimate from the number
+// of outputs alone, which saw neither the channels beyond O of a tile, nor padding slots, nor how rows leave, lost 4.9 % on the
+// mean, more than 5 % in 10 % of the launches and up to a factor of 3.3.
+// E.g. 3x3 with 256 channels at 14x14: batch 4 6.9 us here, 8.1 there; batch 8 8.6 / 8.1; batch 64 42.0 / 10.9.  64 channels at 56x56,
+// batch 64, residual form: 73 / 29 us with rows that start on 32 bytes; on 16 the tensor-core engine stores 4 bytes at a time: 73 / 170.
+double int_pipes_us(dabnn_shape in, int O, dabnn_conv cv, int epi, bool out_nchw, bool vec, int sms) {
+  const int words = (in.C + 63) / 64, ochan = epi == EPI_I32 ? O : (O + 63) / 64 * 64;
+  const long long M = (long long)in.N * dabnn_out_dim(in.H, cv.kh, cv.stride_h, cv.pad_h) * dabnn_out_dim(in.W, cv.kw, cv.stride_w, cv.pad_w);
+  const long long K64 = (long long)words * cv.kh * cv.kw;
+  const int tile = choose_tile(M, ochan, K64, sms);
+  const int bp = tile == 2 ? 128 : tile == 3 ? 64 : tile == 4 ? 32 : 16, bo = tile <= 3 ? 64 : 32;
+  const long long ctas = tile_ctas(M, ochan, bp, bo), slots = (long long)sms * (tile <= 3 ? 2 : 4);
+  // (million outputs, those of ragged tiles included; a last round that is nearly empty counts by 30 %)
+  const double computed = 1e-6 * bp * bo * (tile == 5 ? (double)ctas : 0.7 * ctas + 0.3 * ((ctas + slots - 1) / slots * slots));
+  const double outputs = 1e-6 * M * O;
+  const double per_mac = (tile == 2 ? 0.245 : tile == 3 ? 0.266 : tile == 4 ? 0.272 : 0.097) + (words % 2 ? 0.020 : 0.0);
+  const double per_out = (tile == 2 ? 0.97 : tile == 3 ? 0.79 : tile == 4 ? 1.96 : 3.16) + (words % 2 ? 0.33 : 0.0);
+  double us = 2.1 + (per_mac * K64 + per_out) * computed + (tile <= 3 ? 2.3 : tile == 4 ? 0.0225 * K64 : 0.057 * K64);
+  const bool pieces = vec && O % 4 == 0;  // rows leave in 16-byte pieces
+  if (epi == EPI_I32) us += (out_nchw ? 0.80 : pieces ? 0.0 : 0.44) * outputs;
+  if (epi == EPI_BIREAL) us += (pieces ? 1.77 : 2.73) * outputs;
+  return us;
+}
 
 int sm_count() {
   static int cached[kMaxDevices] = {};
@@ -237,8 +265,10 @@ extern "C" dabnn_status dabnn_bconv2d(const uint64_t* a_packed, dabnn_shape in, 
   if (!out) return DABNN_ERR_NULL;
   if (out_layout != DABNN_NCHW && out_layout != DABNN_NHWC) return DABNN_ERR_SHAPE;
   if (!aligned(out, 4)) return DABNN_ERR_ALIGNMENT;
-  if (tensor_route(in, w_packed, O, cv, EPI_I32)) {
-    s = tc_bits_bconv2d(a_packed, in, w_packed, O, cv, out, out_layout == DABNN_NCHW, as_stream(stream));
+  if (tensor_route(w_packed)) {
+    const bool nchw = out_layout == DABNN_NCHW;
+    const int sms = sm_count();
+    s = tc_bits_bconv2d(a_packed, in, w_packed, O, cv, out, nchw, int_pipes_us(in, O, cv, EPI_I32, nchw, aligned(out, 16), sms), sms, as_stream(stream));
     if (s != DABNN_ERR_UNSUPPORTED) return s;
   }
   g.out = out;
@@ -268,8 +298,10 @@ extern "C" dabnn_status dabnn_bconv2d_bn_sign_pack(const uint64_t* a_packed, dab
   if (s != DABNN_OK) return s;
   if (!scale || !shift || !out_packed) return DABNN_ERR_NULL;
   if (!aligned(scale, 4) || !aligned(shift, 4) || !aligned(out_packed, 8)) return DABNN_ERR_ALIGNMENT;
-  if (tensor_route(in, w_packed, O, cv, EPI_BNPACK)) {
-    s = tc_bits_bn_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, out_packed, as_stream(stream));
+  if (tensor_route(w_packed)) {
+    const int sms = sm_count();
+    s = tc_bits_bn_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, out_packed,
+                             int_pipes_us(in, O, cv, EPI_BNPACK, false, true, sms), sms, as_stream(stream));
     if (s != DABNN_ERR_UNSUPPORTED) return s;
   }
   g.scale = scale; g.shift = shift;
@@ -279,8 +311,9 @@ extern "C" dabnn_status dabnn_bconv2d_bn_sign_pack(const uint64_t* a_packed, dab
 
 extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in,
                                                        const uint64_t* w_packed, int O, dabnn_conv cv,
-                                                       const float* scale, const float* shift, const float* residual,
-                                                       float* y_out, uint64_t* out_packed, void* stream) {
+                                                       const float* scale, const float* shift,
+                                                       const float* residual, float* y_out, uint64_t* out_packed,
+                                                       void* stream) {
   BConvArgs g;
   dabnn_status s = fill_args(g, a_packed, in, w_packed, O, cv);
   if (s != DABNN_OK) return s;
@@ -288,8 +321,10 @@ extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed,
   if (!aligned(scale, 4) || !aligned(shift, 4) || !aligned(residual, 4) || !aligned(y_out, 4) ||
       !aligned(out_packed, 8))
     return DABNN_ERR_ALIGNMENT;
-  if (tensor_route(in, w_packed, O, cv, EPI_BIREAL)) {
-    s = tc_bits_bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed, as_stream(stream));
+  if (tensor_route(w_packed) && !g_chain_launch) {  // (in a chained forward: a block whose caller gave no prepared weights)
+    const int sms = sm_count();
+    s = tc_bits_bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed,
+                                 int_pipes_us(in, O, cv, EPI_BIREAL, false, aligned(residual, 16) && aligned(y_out, 16), sms), sms, as_stream(stream));
     if (s != DABNN_ERR_UNSUPPORTED) return s;
   }
   g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;

@@ -35,6 +35,8 @@
 // Every wait on an mbarrier is bounded: on expiry the kernel records an error flag, stops, frees its TMEM and returns.
 #include "common.cuh"
 
+#include <atomic>
+
 #include <cuda.h>  // the tensor-map type and enums only: the one driver function used is looked up at run time
 
 namespace dabnn {
@@ -57,10 +59,12 @@ constexpr int TC_TMEM_COLS = 512;         // the accumulators' columns + the sca
 constexpr int TC_WAIT_POLLS = 1 << 20;    // polls of a barrier wait before it gives up (about a second)
 constexpr int TC_ACC_COLS = 384;          // columns [0, 384): up to four accumulators (three of 128 columns)
 constexpr int TC_SF_COL = 384;            // columns [384, 512) hold scale factors (all 1.0)
+constexpr double TC_LEAST_US = 4.8;        // no launch is estimated to take less
 constexpr int TC_MAX_BUFS = 4;            // accumulators / activation buffers in flight at most
 
 __device__ int g_tc_error = 0;  // 1: an mbarrier wait ran out (one copy per device; cleared when read by dabnn_last_device_flag)
 int g_tc_max_ctas = 0;          // host: CTAs per launch at most (0: one per SM)
+std::atomic<unsigned long long> g_tc_launches{0};  // host: launches of this engine so far
 
 struct TcArgs {
   const uint64_t* a;
@@ -1192,6 +1196,12 @@ int tc_ntile(int O, int C, int taps, bool pair) {
 // Channel tiles cover O rounded up to whole 64-bit sign words (rows beyond O hold zero weights).
 int tc_n_ntiles(int O, int nt) { return ((O + 63) / 64 * 64 + nt - 1) / nt; }
 
+dabnn_status tc_launched() {
+  const dabnn_status s = launch_status();
+  if (s == DABNN_OK) g_tc_launches.fetch_add(1, std::memory_order_relaxed);
+  return s;
+}
+
 template <int NT, int EPI, int SPT, bool PAIR, bool RES_TMA = false, bool KG = false, int CWX = 0>
 dabnn_status tc_launch(const TcArgs& g, size_t smem, cudaStream_t st) {
   auto kern = bconv_tc_kernel<NT, EPI, SPT, PAIR, RES_TMA, KG, CWX>;
@@ -1240,7 +1250,7 @@ dabnn_status tc_launch(const TcArgs& g, size_t smem, cudaStream_t st) {
   if (units > cap) units = cap;
   if (!PAIR && !g.chained) {
     kern<<<(unsigned)units, TC_THREADS, smem, st>>>(g);
-    return launch_status();
+    return tc_launched();
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((PAIR ? 2 : 1) * units));
@@ -1264,7 +1274,7 @@ dabnn_status tc_launch(const TcArgs& g, size_t smem, cudaStream_t st) {
     cudaGetLastError();
     return DABNN_ERR_CUDA;
   }
-  return launch_status();
+  return tc_launched();
 }
 
 // cuTensorMapEncodeTiled, looked up through the runtime (the library does not link against the driver library)
@@ -1399,12 +1409,13 @@ dabnn_status tc_dispatch_mode(TcArgs& g, cudaStream_t st) {
   return DABNN_ERR_UNSUPPORTED;
 }
 
-void tc_plan(TcArgs& g, int epi);
+double tc_plan(TcArgs& g, int epi, int sms);
 
+// limit_us: what the caller's other engine would take; a launch that is estimated to take longer here is left to it.
 template <int EPI>
-dabnn_status tc_dispatch(TcArgs& g, cudaStream_t st) {
-  tc_plan(g, EPI);
-  if (g.ntile == 0) return DABNN_ERR_UNSUPPORTED;
+dabnn_status tc_dispatch(TcArgs& g, cudaStream_t st, double limit_us = 1e300, int sms = 0) {
+  const double us = tc_plan(g, EPI, sms != 0 ? sms : sm_count());
+  if (g.ntile == 0 || us >= limit_us) return DABNN_ERR_UNSUPPORTED;
   // A second group of epilogue warps (measured): it pays for the residual epilogue, which moves two fp32 rows per
   // output row; elsewhere the extra warps only add contention.
   // (environment DABNN_TC_EPI2 = 0 / 1 overrides, for measurements)
@@ -1425,13 +1436,13 @@ bool tc_wide_rows(const TcArgs& g, int epi) {
   return epi == EPI_I32 ? aligned(g.out, 32) : aligned(g.residual, 32) && aligned(g.y_out, 32);
 }
 
-// Launch form for a problem: CTA pairs when there are enough tiles to fill the chip with pairs, and as many channel
-// tiles resident per CTA (pair) as fit while every CTA (pair) still gets work.
-void tc_plan(TcArgs& g, int epi) {
+// Launch form for a problem: CTA pairs when there are enough tiles to fill the chip with pairs, and the number of channel tiles
+// resident per CTA (pair).  Returns the estimated time of the launch in microseconds.
+double tc_plan(TcArgs& g, int epi, int sms) {
   const int O = g.O, C = g.C, taps = g.kh * g.kw;
   const long long Kb = (long long)tc_cpad(C) / 2 * taps;
   const int mode = tc_mode();
-  const int units1 = sm_count(), units2 = sm_count() / 2;
+  const int units1 = sms, units2 = sms / 2;
   const int nt2 = tc_ntile(O, C, taps, true);
   bool pair = nt2 != 0 && mode != 1 && g.kgroups == 1;
   if (pair && mode == 0) {
@@ -1442,7 +1453,7 @@ void tc_plan(TcArgs& g, int epi) {
   }
   g.pair = pair ? 1 : 0;
   g.ntile = pair ? nt2 : tc_ntile(O, C, taps, false);
-  if (g.ntile == 0) return;
+  if (g.ntile == 0) return 0;
   g.n_ntiles = tc_n_ntiles(O, g.ntile);
   const long long wr = pair ? g.ntile / 2 : g.ntile;
   long long nres = TC_WEIGHT_BUDGET / (wr * Kb);
@@ -1467,6 +1478,7 @@ void tc_plan(TcArgs& g, int epi) {
   const long long most = pair ? units2 - 8 : units1;
   long long best = -1;
   int best_n = (int)nres;
+  long long best_rounds = m_units;
   for (int n = (int)nres; n >= 1; n--) {
     const long long groups = (g.n_ntiles + n - 1) / n;
     if (groups > most) break;
@@ -1480,11 +1492,30 @@ void tc_plan(TcArgs& g, int epi) {
     if (best < 0 || cost < best) {
       best = cost;
       best_n = n;
+      best_rounds = rounds;
     }
   }
   nres = best_n;
   g.nres = (int)nres;
   g.n_groups = (g.n_ntiles + g.nres - 1) / g.nres;
+  // The estimate, fitted (least squares of the relative error; 90 % of the launches within -27 and +18 %) to 1619 launches: 1 to
+  // 9216 channels, filters of 1 to 9 rows and columns, strides 1 and 2, images of 1 to 224 pixels a side, O 1 to 4096, every output
+  // form, outputs at 4-, 8-, 16- and 32-byte offsets.
+  const double live = (double)(nres * g.ntile < o_cols ? nres * g.ntile : o_cols) / 128;
+  const double outputs = 1e-6 * g.N * g.OH * g.OW * O;
+  const double main_cyc = (double)(nres * mma_cyc > exp_cyc ? nres * mma_cyc : exp_cyc);
+  double per_tile = 1.36e-3 / 1.9 * main_cyc + 0.26, rest = TC_LEAST_US + 0.9 * nres * wr * Kb / 40 / 1.9e3;
+  if (epi == EPI_BNPACK) {
+    per_tile += 0.51 * live;
+  } else if (epi == EPI_I32) {
+    per_tile += (wide ? 0.68 : 1.9) * live;
+    rest += (g.out_nchw ? 1.64 : wide ? 0.08 : 4.0) * outputs;
+  } else {
+    per_tile += (wide ? 0.53 : 9.6) * live;
+    rest += (wide ? 0.89 : 7.3) * outputs + 0.8;
+  }
+  // (4-byte stores: the spread of the estimate is wider, and the other engine's time the surer one)
+  return (wide ? 1.0 : 1.05) * (rest + best_rounds * per_tile);
 }
 
 // w: packed words at a 16-byte boundary (a prepared buffer, or the caller's packed weights where they start on one)
@@ -1535,35 +1566,6 @@ dabnn_status tc_fill(TcArgs& g, const uint64_t* a, dabnn_shape in, const void* w
 
 }  // namespace
 
-// Packed-weight calls (epi: the output form) that run on this engine: where its estimated time is below that of the
-// xor/popcount kernel.  Both estimates are fits, in microseconds, to back-to-back launches on a B200 over 8 to 17 layer
-// shapes (C 16 to 512, 1x1 and 3x3, stride 1 and 2, O 16 to 2048) at batch 1 to 256:
-//   xor/popcount: 3.5 + 0.43 per million word multiply-adds + 0.9 per million outputs (2.1 where a row is an odd number of
-//     words and is loaded in 8-byte pieces); the forms with sign words work on whole words of 64 channels
-//   tensor: 6 + up to 3 for expanding the resident weights + 0.07 per million word multiply-adds + 0.9 per million outputs
-//     (sign words 0.3); stride 2 +0.7, with C > 128 +2.3 more (one activation buffer, filled after the weights are expanded);
-//     the residual stream +1.5; outputs whose rows are not whole 32-byte pieces leave by 4-byte stores: +4 per million int32,
-//     +24 per million residual outputs
-// E.g. 3x3 with 256 channels at 14x14: batch 4 6.9 against 8.6 us, batch 8 8.6 / 8.7, batch 16 14.2 / 8.8, batch 64 42.0 / 11.5;
-// 64 channels at 56x56: batch 4 6.9 / 5.9, batch 64 51.6 / 17.1.
-bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi, double hidden) {
-  if (cv.stride_h != cv.stride_w || cv.stride_h > 2 || !tc_covers(O, in.C, cv.kh * cv.kw)) return false;
-  const int taps = cv.kh * cv.kw, nt = tc_ntile(O, in.C, taps, false);
-  if (nt == 0) return false;
-  const double words = (in.C + 63) / 64;
-  const double outputs = (double)in.N * dabnn_out_dim(in.H, cv.kh, cv.stride_h, cv.pad_h) *
-                         dabnn_out_dim(in.W, cv.kw, cv.stride_w, cv.pad_w) * O * 1e-6;
-  const double macs = outputs * words * taps;
-  const double weights = (double)(O < nt ? O : nt) * tc_cpad(in.C) / 2 * taps / TC_WEIGHT_BUDGET;
-  const double whole = epi == EPI_I32 ? 1.0 : (double)((O + 63) / 64 * 64) / O;
-  const double t_int = 3.5 + whole * (0.43 * macs + (((in.C + 63) / 64 * taps) % 2 ? 2.1 : 0.9) * outputs);
-  double t_tc = 6.0 + 3.0 * weights + 0.07 * macs + (epi == EPI_BNPACK ? 0.3 : 0.9) * outputs;
-  if (cv.stride_h == 2) t_tc += in.C > 128 ? 3.0 : 0.7;
-  if (epi == EPI_BIREAL) t_tc += 1.5;
-  if (O % 8 != 0) t_tc += (epi == EPI_I32 ? 4.0 : epi == EPI_BIREAL ? 24.0 : 0.0) * outputs;
-  return t_tc - hidden < t_int;
-}
-
 }  // namespace dabnn
 
 using namespace dabnn;
@@ -1612,39 +1614,43 @@ extern "C" dabnn_status dabnn_tc_bconv2d_bn_sign_pack(const uint64_t* a_packed, 
 
 namespace dabnn {
 dabnn_status tc_bits_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv, int32_t* out,
-                             bool out_nchw, cudaStream_t st) {
+                             bool out_nchw, double limit_us, int sms, cudaStream_t st) {
+  if (limit_us <= TC_LEAST_US) return DABNN_ERR_UNSUPPORTED;
   TcArgs g;
   dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
   if (s != DABNN_OK) return s;
   g.out = out;
   g.out_nchw = out_nchw;
-  return tc_dispatch<EPI_I32>(g, st);
+  return tc_dispatch<EPI_I32>(g, st, limit_us, sms);
 }
 
 dabnn_status tc_bits_bn_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
-                                  const float* scale, const float* shift, uint64_t* out_packed, cudaStream_t st) {
+                                  const float* scale, const float* shift, uint64_t* out_packed, double limit_us, int sms, cudaStream_t st) {
+  if (limit_us <= TC_LEAST_US) return DABNN_ERR_UNSUPPORTED;
   TcArgs g;
   dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
   if (s != DABNN_OK) return s;
   g.scale = scale; g.shift = shift;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
-  return tc_dispatch<EPI_BNPACK>(g, st);
+  return tc_dispatch<EPI_BNPACK>(g, st, limit_us, sms);
 }
 
 dabnn_status tc_bits_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
                                       const float* scale, const float* shift, const float* residual, float* y_out,
-                                      uint64_t* out_packed, cudaStream_t st) {
+                                      uint64_t* out_packed, double limit_us, int sms, cudaStream_t st) {
+  if (limit_us <= TC_LEAST_US) return DABNN_ERR_UNSUPPORTED;
   TcArgs g;
   dabnn_status s = tc_fill(g, a_packed, in, w_packed, O, cv);
   if (s != DABNN_OK) return s;
   g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
-  return tc_dispatch<EPI_BIREAL>(g, st);
+  return tc_dispatch<EPI_BIREAL>(g, st, limit_us, sms);
 }
 
 dabnn_status tc_bireal_block(const uint64_t* a_packed, dabnn_shape in, const void* w_tc, int O, dabnn_conv cv,
                              const float* scale, const float* shift, const float* residual, float* y_out,
-                             uint64_t* out_packed, bool chained, cudaStream_t st) {
+                             uint64_t* out_packed, bool chained, double limit_us, int sms, cudaStream_t st) {
+  if (limit_us <= TC_LEAST_US) return DABNN_ERR_UNSUPPORTED;
   TcArgs g;
   dabnn_status s = tc_fill(g, a_packed, in, w_tc, O, cv);
   if (s != DABNN_OK) return s;
@@ -1654,7 +1660,7 @@ dabnn_status tc_bireal_block(const uint64_t* a_packed, dabnn_shape in, const voi
   g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
   g.chained = chained ? 1 : 0;
-  return tc_dispatch<EPI_BIREAL>(g, st);
+  return tc_dispatch<EPI_BIREAL>(g, st, limit_us, sms);
 }
 }  // namespace dabnn
 
@@ -1687,6 +1693,8 @@ extern "C" int dabnn_tc_set_max_ctas(int max_ctas) {
   g_tc_max_ctas = max_ctas > 0 ? max_ctas : 0;
   return prev;
 }
+
+extern "C" unsigned long long dabnn_tc_launches(void) { return g_tc_launches.load(std::memory_order_relaxed); }
 
 extern "C" int dabnn_tc_error_flag(void) {
   int v = 0;

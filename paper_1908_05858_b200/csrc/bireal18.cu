@@ -889,6 +889,7 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
   }
   // consecutive tensor-engine blocks are chained (DABNN_NO_CHAIN=1 keeps the ordinary stream order)
   const bool tc_chain = !chain_off;
+  const int sms = sm_count();
   int C = 64, HW = 56;
   for (int b = 0; b < 16; b++) {
     const int stage = b / 4, O = kStageC[stage], OHW = kStageHW[stage];
@@ -918,9 +919,9 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
     // tensor-core engine where it covers the layer and pays; chained launches hide part of its start-up (measured: a credit
     // of 1.5 us against lone launches; batch 8 240 -> 234 us, batch 12 283 -> 269, batch 16 340 -> 322, batch 4 unchanged;
     // with 3 us batch 2 and 4 lose 3 us each)
-    if (p->block_w_tc[b] != nullptr && tc_bits_worthwhile(in, O, cv, 2, tc_chain ? 1.5 : 0.0))
+    if (p->block_w_tc[b] != nullptr)
       s = tc_bireal_block(bits_in, in, p->block_w_tc[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
-                          b == 15 ? nullptr : bits_out, tc_chain, st);
+                          b == 15 ? nullptr : bits_out, tc_chain, int_pipes_us(in, O, cv, 2, false, true, sms) + (tc_chain ? 1.5 : 0.0), sms, st);
     if (s == DABNN_ERR_UNSUPPORTED)
       s = dabnn_bconv2d_bn_add_sign_pack(bits_in, in, p->block_w[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
                                          b == 15 ? nullptr : bits_out, st);

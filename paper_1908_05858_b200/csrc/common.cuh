@@ -17,25 +17,27 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 inline int ceil_div(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
 
-// Layers (epi: 0 int32, 1 sign words, 2 residual stream) that are faster on the tensor-core engine than on the integer pipes;
-// hidden: microseconds of its start-up that pass under a previous kernel.
-bool tc_bits_worthwhile(dabnn_shape in, int O, dabnn_conv cv, int epi, double hidden = 0.0);
+// Estimated time, in microseconds, of a layer on the integer pipes (epi: 0 int32, 1 sign words, 2 residual stream; vec: the fp32 or
+// int32 rows start on 16 bytes; sms: sm_count(), which asks the runtime and is asked once per call).
+double int_pipes_us(dabnn_shape in, int O, dabnn_conv cv, int epi, bool out_nchw, bool vec, int sms);
 
 // The three output forms on the tensor-core engine from the caller's packed weights (16-byte aligned).  Arguments as of the
-// entry points of the same form, already checked; DABNN_ERR_UNSUPPORTED where the engine does not cover the layer.
+// entry points of the same form, already checked; DABNN_ERR_UNSUPPORTED where the engine does not cover the layer or is estimated
+// to take longer than limit_us.
 dabnn_status tc_bits_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv, int32_t* out,
-                             bool out_nchw, cudaStream_t st);
+                             bool out_nchw, double limit_us, int sms, cudaStream_t st);
 dabnn_status tc_bits_bn_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
-                                  const float* scale, const float* shift, uint64_t* out_packed, cudaStream_t st);
+                                  const float* scale, const float* shift, uint64_t* out_packed, double limit_us, int sms, cudaStream_t st);
 dabnn_status tc_bits_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
                                       const float* scale, const float* shift, const float* residual, float* y_out,
-                                      uint64_t* out_packed, cudaStream_t st);
+                                      uint64_t* out_packed, double limit_us, int sms, cudaStream_t st);
 
 // The Bi-Real block on the tensor-core engine as the forward launches it.  chained: with programmatic stream serialization
 // (the kernel sets itself up under its predecessor's tail; its weights and BN vectors must be constants of the stream).
+// limit_us as above.
 dabnn_status tc_bireal_block(const uint64_t* a_packed, dabnn_shape in, const void* w_tc, int O, dabnn_conv cv,
                              const float* scale, const float* shift, const float* residual, float* y_out,
-                             uint64_t* out_packed, bool chained, cudaStream_t st);
+                             uint64_t* out_packed, bool chained, double limit_us, int sms, cudaStream_t st);
 
 // Chained launches for forwards of a few images, where every kernel is shorter than the time it takes to start one.  A
 // kernel started by launch_chain() while g_chain_launch is set may begin before its predecessor in the stream has

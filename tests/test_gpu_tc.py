@@ -467,3 +467,57 @@ def test_packed_weight_calls_on_this_engine_match_oracle(B, oracle_mod, case):
         assert np.array_equal(got_y.cpu().numpy().view(np.uint32), y.view(np.uint32))
         assert np.array_equal(u64(got_ybits), want_ybits)
     assert B.last_device_flag() == 0
+
+
+def placed(shape, dtype, offset):
+    """A tensor whose first byte lies `offset` bytes beyond a 256-byte boundary."""
+    n = int(np.prod(shape)) * torch.empty((), dtype=dtype).element_size()
+    raw = torch.full((n + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    assert raw.data_ptr() % 256 == 0
+    return raw[offset:offset + n].view(dtype).view(shape)
+
+
+# Which engine a packed-weight call takes follows what that engine will really do: rows that do not start on 32 bytes (or are no
+# multiple of 32 bytes) leave it by 4-byte stores, small padded images are mostly padding slots to it, and the integer pipes
+# compute whole tiles of 64 channels whatever O is.
+ROUTE_CASES = [
+    # N, C, H, W, O, k, pad, pad_value, stride; byte offset of int32 sums, residual; int32 / sign words / residual on this engine
+    ((24, 64, 56, 56, 64, 3, 1, -1, 1), 0, (True, True, True)),
+    ((24, 64, 56, 56, 64, 3, 1, -1, 1), 4, (False, True, False)),
+    ((24, 64, 56, 56, 64, 3, 1, -1, 1), 8, (False, True, False)),
+    ((24, 64, 56, 56, 64, 3, 1, +1, 1), 16, (False, True, False)),
+    ((30, 256, 14, 14, 256, 3, 1, -1, 1), 16, (True, True, False)),
+    ((16, 51, 56, 59, 353, 3, 1, -1, 1), 0, (False, True, False)),
+    ((600, 21, 3, 3, 21, 7, 3, -1, 1), 0, (False, False, False)),
+    ((30, 64, 56, 56, 1, 3, 1, -1, 1), 0, (True, True, True)),
+    ((2, 64, 14, 14, 64, 3, 1, -1, 1), 0, (False, False, False)),
+]
+
+
+@pytest.mark.parametrize("case,offset,here", ROUTE_CASES)
+def test_packed_weight_calls_take_the_faster_engine(B, oracle_mod, case, offset, here):
+    N, C, H, W, O, k, pad, pv, s = case
+    x, w = inputs(case)
+    o = oracle_mod
+    st = (s, s)
+    acc = o.bconv_bits(o.pack(x), C, o.pack_weights(w), st, (pad, pad), pv, o.NHWC)
+    rng = np.random.default_rng(O + N)
+    scale, shift = o.bn_fold(*synth.bn_params(rng, O))
+    res = (rng.standard_normal(acc.shape) * 15).astype(np.float32)
+    y, want_ybits = o.bn_add_sign_pack(acc, scale, shift, res)
+    a, wp = B.pack(dev(x)), B.pack_weights(dev(w))
+    n0 = B.tc_launches()
+    got = B.bconv2d(a, C, wp, st, (pad, pad), pv, out=placed(acc.shape, torch.int32, offset))
+    n1 = B.tc_launches()
+    bits = B.bconv2d_bn_sign_pack(a, C, wp, dev(scale), dev(shift), st, (pad, pad), pv)
+    n2 = B.tc_launches()
+    residual = placed(acc.shape, torch.float32, offset)
+    residual.copy_(dev(res))
+    got_y, got_ybits = B.bconv2d_bn_add_sign_pack(a, C, wp, dev(scale), dev(shift), residual, st, (pad, pad), pv)
+    n3 = B.tc_launches()
+    assert (n1 - n0, n2 - n1, n3 - n2) == tuple(int(h) for h in here)
+    assert np.array_equal(got.cpu().numpy(), acc)
+    assert np.array_equal(u64(bits), o.bn_sign_pack(acc, scale, shift))
+    assert np.array_equal(got_y.cpu().numpy().view(np.uint32), y.view(np.uint32))
+    assert np.array_equal(u64(got_ybits), want_ybits)
+    assert B.last_device_flag() == 0
