@@ -148,7 +148,8 @@ typedef struct {
   const void* block_w_tc[16];    /* optional: weights prepared by dabnn_tc_prepare_weights, or NULL.  Where given and the
                                     layer is large enough to be faster on the tensor-core engine
                                     (the early stages from 4 images, all blocks from about 64), that engine runs the
-                                    block; results are identical either way */
+                                    block; where it is NULL the integer pipes do, whatever the size; results are
+                                    identical either way */
 } dabnn_bireal18_params;
 
 /* Bytes of device workspace dabnn_bireal18_forward needs for a batch of N images (0 if N <= 0). */

@@ -309,11 +309,9 @@ extern "C" dabnn_status dabnn_bconv2d_bn_sign_pack(const uint64_t* a_packed, dab
   return launch_epi<EPI_BNPACK>(g, as_stream(stream));
 }
 
-extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in,
-                                                       const uint64_t* w_packed, int O, dabnn_conv cv,
-                                                       const float* scale, const float* shift,
-                                                       const float* residual, float* y_out, uint64_t* out_packed,
-                                                       void* stream) {
+static dabnn_status bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                     const float* scale, const float* shift, const float* residual, float* y_out,
+                                     uint64_t* out_packed, bool either_engine, cudaStream_t st) {
   BConvArgs g;
   dabnn_status s = fill_args(g, a_packed, in, w_packed, O, cv);
   if (s != DABNN_OK) return s;
@@ -321,15 +319,29 @@ extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed,
   if (!aligned(scale, 4) || !aligned(shift, 4) || !aligned(residual, 4) || !aligned(y_out, 4) ||
       !aligned(out_packed, 8))
     return DABNN_ERR_ALIGNMENT;
-  if (tensor_route(w_packed) && !g_chain_launch) {  // (in a chained forward: a block whose caller gave no prepared weights)
+  if (either_engine && tensor_route(w_packed)) {
     const int sms = sm_count();
     s = tc_bits_bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed,
-                                 int_pipes_us(in, O, cv, EPI_BIREAL, false, aligned(residual, 16) && aligned(y_out, 16), sms), sms, as_stream(stream));
+                                 int_pipes_us(in, O, cv, EPI_BIREAL, false, aligned(residual, 16) && aligned(y_out, 16), sms), sms, st);
     if (s != DABNN_ERR_UNSUPPORTED) return s;
   }
   g.scale = scale; g.shift = shift; g.residual = residual; g.y_out = y_out;
   g.out_packed32 = reinterpret_cast<uint32_t*>(out_packed);
-  return launch_epi<EPI_BIREAL>(g, as_stream(stream));
+  return launch_epi<EPI_BIREAL>(g, st);
+}
+
+dabnn_status dabnn::int_pipes_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                               const float* scale, const float* shift, const float* residual, float* y_out,
+                                               uint64_t* out_packed, cudaStream_t st) {
+  return bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed, false, st);
+}
+
+extern "C" dabnn_status dabnn_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in,
+                                                       const uint64_t* w_packed, int O, dabnn_conv cv,
+                                                       const float* scale, const float* shift,
+                                                       const float* residual, float* y_out, uint64_t* out_packed,
+                                                       void* stream) {
+  return bn_add_sign_pack(a_packed, in, w_packed, O, cv, scale, shift, residual, y_out, out_packed, true, as_stream(stream));
 }
 
 extern "C" dabnn_status dabnn_bgemm(const uint64_t* A, int M, const uint64_t* B, int N, int Kbits, int32_t* C,

@@ -923,8 +923,8 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
       s = tc_bireal_block(bits_in, in, p->block_w_tc[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
                           b == 15 ? nullptr : bits_out, tc_chain, int_pipes_us(in, O, cv, 2, false, true, sms) + (tc_chain ? 1.5 : 0.0), sms, st);
     if (s == DABNN_ERR_UNSUPPORTED)
-      s = dabnn_bconv2d_bn_add_sign_pack(bits_in, in, p->block_w[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
-                                         b == 15 ? nullptr : bits_out, st);
+      s = int_pipes_bn_add_sign_pack(bits_in, in, p->block_w[b], O, cv, p->block_scale[b], p->block_shift[b], cur, cur,
+                                     b == 15 ? nullptr : bits_out, st);
     if (s != DABNN_OK) return s;
     uint64_t* tb = bits_in; bits_in = bits_out; bits_out = tb;
     C = O; HW = OHW;

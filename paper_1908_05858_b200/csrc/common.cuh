@@ -32,6 +32,11 @@ dabnn_status tc_bits_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, 
                                       const float* scale, const float* shift, const float* residual, float* y_out,
                                       uint64_t* out_packed, double limit_us, int sms, cudaStream_t st);
 
+// dabnn_bconv2d_bn_add_sign_pack on the integer pipes whatever the size: a forward's block whose caller gave no prepared weights.
+dabnn_status int_pipes_bn_add_sign_pack(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
+                                        const float* scale, const float* shift, const float* residual, float* y_out,
+                                        uint64_t* out_packed, cudaStream_t st);
+
 // The Bi-Real block on the tensor-core engine as the forward launches it.  chained: with programmatic stream serialization
 // (the kernel sets itself up under its predecessor's tail; its weights and BN vectors must be constants of the stream).
 // limit_us as above.

@@ -521,3 +521,33 @@ def test_packed_weight_calls_take_the_faster_engine(B, oracle_mod, case, offset,
     assert np.array_equal(got_y.cpu().numpy().view(np.uint32), y.view(np.uint32))
     assert np.array_equal(u64(got_ybits), want_ybits)
     assert B.last_device_flag() == 0
+
+
+_NO_CHAIN_SCRIPT = r"""
+import sys, numpy as np, torch
+from paper_1908_05858_b200 import binding as B, synth
+p = synth.bireal18_params()
+img = torch.from_numpy(synth.bireal18_images(16)).cuda()
+n0 = B.tc_launches()
+popc = B.Bireal18(p, engine="popc").forward(img).cpu().numpy()
+n1 = B.tc_launches()
+auto = B.Bireal18(p).forward(img).cpu().numpy()
+n2 = B.tc_launches()
+assert n1 == n0, "a forward without prepared weights ran %d blocks on the tensor-core engine" % (n1 - n0)
+assert n2 > n1
+assert np.array_equal(popc.view(np.uint32), auto.view(np.uint32)) and B.last_device_flag() == 0
+print("engines ok")
+"""
+
+
+@pytest.mark.parametrize("no_chain", [False, True])
+def test_a_forward_without_prepared_weights_stays_on_the_integer_pipes(no_chain):
+    """DABNN_NO_CHAIN (read once per process) changes the order of launches, not the engine."""
+    import os, subprocess, sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, PYTHONPATH=root + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    env.pop("DABNN_NO_CHAIN", None)
+    if no_chain:
+        env["DABNN_NO_CHAIN"] = "1"
+    r = subprocess.run([sys.executable, "-c", _NO_CHAIN_SCRIPT], env=env, cwd=root, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "engines ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
