@@ -28,8 +28,8 @@
  *     work, so they still return DABNN_OK then; read the flag with dabnn_stream_status / dabnn_last_device_flag.
  *   - Devices: a process may use the library on several devices (cudaSetDevice before the call); caches of function
  *     attributes and SM counts are kept per device ordinal (up to 64).
- *   - Alignment: packed buffers 8 bytes; fp32 buffers 4 bytes (16 bytes enables vector paths,
- *     chosen automatically).
+ *   - Alignment: packed buffers 8 bytes; fp32 and int32 buffers 4 bytes (16 bytes, and for the tensor-core engine's outputs 32,
+ *     enable vector paths, chosen automatically).
  */
 #ifndef DABNN_H_
 #define DABNN_H_
@@ -97,10 +97,11 @@ dabnn_status dabnn_pack_weights(const float* w_oihw, int O, int C, int kh, int k
 
 /* Section 2.1.2, Eq. 1 -- binary convolution, int32 result.
  * a_packed: [N][H][W][Cw] for in = {N,C,H,W}; w_packed: [O][kh][kw][Cw];
- * (These calls and the fused forms below run on the integer pipes or, where a launch is large enough to be faster there and
- * w_packed is 16-byte aligned, on the tensor-core engine: same integers; see dabnn_last_device_flag for that engine's
- * bounded waits, and dabnn_set_conv_variant / dabnn_set_conv_tile to keep a measurement on the integer pipes.)
- * out: int32, N*OH*OW*O elements in `out_layout` ([N][OH][OW][O] or [N][O][OH][OW]). */
+ * out: int32, N*OH*OW*O elements in `out_layout` ([N][OH][OW][O] or [N][O][OH][OW]).
+ * This call, dabnn_bgemm and the fused forms below run on the integer pipes or, where a launch is estimated to be faster there
+ * and w_packed is 16-byte aligned, on the tensor-core engine: the same integers.  That engine stores whole rows where they
+ * are multiples of 32 bytes at 32-byte aligned addresses.  Its waits are bounded, so after synchronising check
+ * dabnn_stream_status.  dabnn_set_conv_variant / dabnn_set_conv_tile keep a measurement on the integer pipes. */
 dabnn_status dabnn_bconv2d(const uint64_t* a_packed, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
                            int32_t* out, dabnn_layout out_layout, void* stream);
 
@@ -221,8 +222,10 @@ dabnn_status dabnn_bireal18_forward_static(const dabnn_bireal18_params* p, const
  * workspace waits for whatever `stream` held when the function was called whenever the workspace is not the one of the
  * previous call on this device; with the same workspace it waits only for that previous call's kernels, so a caller
  * that lets other work use the workspace in between must synchronise that work itself.  Not thread-safe against
- * concurrent calls on the same device; calls that share a workspace belong on one stream.  This entry point uses the
- * integer-pipe kernels only (no bounded waits), so there is no device flag to read after it. */
+ * concurrent calls on the same device; calls that share a workspace belong on one stream.  Chunks large enough to be faster
+ * there run on the tensor-core engine, as dabnn_bconv2d and dabnn_bconv2d_bn_sign_pack do: where a wait inside one of its
+ * kernels runs out, the call has long returned DABNN_OK and the host buffers hold undefined data.  After synchronising
+ * `stream`, the results are valid only if dabnn_stream_status(stream) is DABNN_OK. */
 size_t dabnn_binary_layer_host_workspace_bytes(dabnn_shape in, int O, dabnn_conv cv);
 dabnn_status dabnn_binary_layer_host(const float* x_host, dabnn_shape in, const uint64_t* w_packed, int O, dabnn_conv cv,
                                      const float* scale, const float* shift, int32_t* out_host, uint64_t* bits_host,

@@ -451,7 +451,9 @@ def binary_layer_host(x_host: torch.Tensor, w_packed: torch.Tensor, workspace: t
                       pad_value: int = -1, scale=None, shift=None, out_host: Optional[torch.Tensor] = None,
                       bits_host: Optional[torch.Tensor] = None):
     """dabnn_binary_layer_host: x_host / out_host / bits_host are HOST tensors (pin them for asynchronous
-    copies); w_packed, scale, shift, workspace are device tensors.  Work is enqueued on the current stream."""
+    copies); w_packed, scale, shift, workspace are device tensors.  Work is enqueued on the current stream.  Large chunks run on
+    the tensor-core engine, whose waits are bounded: the host results are valid once `stream_status()` (which synchronises the
+    stream) has returned 0."""
     if x_host.is_cuda or x_host.dtype != torch.float32 or not x_host.is_contiguous():
         raise DabnnError("x_host must be a contiguous fp32 host tensor")
     w = _dev(w_packed, torch.int64, "w_packed")

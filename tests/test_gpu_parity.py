@@ -575,3 +575,27 @@ def test_binary_layer_host_matches_oracle(B, oracle_mod, N, pinned):
         want = o.bconv_bits(o.pack(x), C, o.pack_weights(w), (1, 1), (1, 1), -1, o.NHWC)
         assert np.array_equal(out_h.numpy(), want)
         assert np.array_equal(bits_h.numpy().view(np.uint64), o.bn_sign_pack(want, scale_np, shift_np))
+
+
+@pytest.mark.parametrize("N,O", [(64, 128), (61, 70)])
+def test_binary_layer_host_with_chunks_on_the_tensor_engine(B, oracle_mod, N, O):
+    """Chunks large enough for the tensor-core engine (which the launch count shows): both outputs against the oracle, and the
+    stream's status, which says whether they are valid, read after the call as the interface asks."""
+    o = oracle_mod
+    C, H, W = 128, 28, 28
+    rng = np.random.default_rng(N + O)
+    x = rng.standard_normal((N, C, H, W)).astype(np.float32)
+    w = rng.standard_normal((O, C, 3, 3)).astype(np.float32)
+    scale_np, shift_np = rng.uniform(0.5, 1.5, O).astype(np.float32), rng.normal(0, 5, O).astype(np.float32)
+    wp, scale, shift = B.pack_weights(dev(w)), dev(scale_np), dev(shift_np)
+    ws = torch.empty(B.binary_layer_host_workspace_bytes(N, C, H, W, O, 3, 3, (1, 1), (1, 1), -1), dtype=torch.uint8, device="cuda")
+    xh = torch.from_numpy(x).pin_memory()
+    out_h = torch.empty((N, H, W, O), dtype=torch.int32).pin_memory()
+    bits_h = torch.empty((N, H, W, (O + 63) // 64), dtype=torch.int64).pin_memory()
+    n0 = B.tc_launches()
+    B.binary_layer_host(xh, wp, ws, (1, 1), (1, 1), -1, scale, shift, out_host=out_h, bits_host=bits_h)
+    assert B.tc_launches() - n0 >= 4  # at least the sign words of each chunk
+    assert B.stream_status() == 0
+    want = o.bconv_bits(o.pack(x), C, o.pack_weights(w), (1, 1), (1, 1), -1, o.NHWC)
+    assert np.array_equal(out_h.numpy(), want)
+    assert np.array_equal(bits_h.numpy().view(np.uint64), o.bn_sign_pack(want, scale_np, shift_np))
