@@ -34,13 +34,16 @@ PACK_SHAPES = [
     (3, 256, 56, 56),   # vector path, four warps per pixel group, ragged last tile (3136 = 24.5 * 128)
     (2, 128, 28, 28),   # vector path, two words
     (1, 192, 12, 12),   # three words
-    (2, 70, 7, 5),      # generic path (H*W not a multiple of 4), channel tail
+    (2, 70, 7, 5),      # tile path (H*W and C*H*W no multiples of 4), channel tail
     (1, 1, 1, 1),
     (1, 1000, 2, 2),    # 16 words, tail of 40 bits
     (5, 3, 224, 8),
-    (4, 512, 7, 7),     # tile path: H*W = 49
-    (2, 100, 15, 13),   # tile path, two pixel tiles, channel tail
-    (1, 2100, 3, 3),    # more than 32 words: generic path
+    (4, 512, 7, 7),     # whole-image path: H*W = 49
+    (2, 100, 15, 13),   # whole-image path, channel tail
+    (1, 2100, 3, 3),    # whole-image path, more than 32 words
+    (2, 100, 17, 19),   # tile path: H*W = 323, three pixel tiles, two words, channel tail
+    (2, 70, 15, 13),    # tile path: C*H*W no multiple of 4, two pixel tiles
+    (1, 200, 19, 23),   # tile path, four pixel tiles, four words
     (3, 100, 15, 15),   # whole-image path: H*W = 225, channel tail, a run of 36 * 225 values
     (2, 68, 1, 3),      # whole-image path with four channels in the last word
     (70, 512, 7, 7),    # whole-image path, many CTAs
@@ -58,11 +61,13 @@ def test_pack_nchw(B, oracle_mod, shape):
     assert np.array_equal(got, oracle_mod.pack(x, oracle_mod.NCHW))
 
 
-# (after the first five: the flat-bitmap path -- a last vector of one to three values, several pixel tiles,
-# large tiles, the largest C of the path and one beyond it)
-@pytest.mark.parametrize("shape", [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (1, 3, 3, 4), (4, 31, 17, 128), (1, 1, 1, 1),
-                                   (3, 1, 1, 1), (1, 7, 11, 35), (2, 33, 17, 33), (37, 27, 29, 100), (90, 28, 28, 70), (1, 6, 6, 4090),
-                                   (1, 3, 3, 4099)])
+# whole words of 64; one thread per word (few channels, one beyond the largest of the flat path); the flat-bitmap path: last
+# vectors of one, two and three values, several pixel tiles, large tiles, its largest C
+PACK_NHWC_SHAPES = [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (1, 3, 3, 4), (4, 31, 17, 128), (1, 1, 1, 1), (3, 1, 1, 1),
+                    (1, 7, 11, 35), (1, 7, 9, 35), (2, 33, 17, 33), (37, 27, 29, 100), (90, 28, 28, 70), (1, 6, 6, 4090), (1, 3, 3, 4099)]
+
+
+@pytest.mark.parametrize("shape", PACK_NHWC_SHAPES)
 def test_pack_nhwc(B, oracle_mod, shape):
     rng = np.random.default_rng(sum(shape) + 1)
     x = rng.standard_normal(shape).astype(np.float32)
@@ -80,7 +85,7 @@ def test_pack_i32_nchw(B, oracle_mod, shape):
     assert np.array_equal(got, oracle_mod.pack_i32(x, oracle_mod.NCHW))
 
 
-@pytest.mark.parametrize("shape", [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (4, 31, 17, 128)])
+@pytest.mark.parametrize("shape", PACK_NHWC_SHAPES)
 def test_pack_i32_nhwc(B, oracle_mod, shape):
     rng = np.random.default_rng(sum(shape) + 3)
     x = rng.integers(-50, 50, size=shape).astype(np.int32)
@@ -135,6 +140,14 @@ CONV_CASES = [
 ]
 
 
+@pytest.fixture(params=[0, 2], ids=["either engine", "integer pipes"])
+def conv_variant(B, request):
+    """0: the library chooses the engine (large calls run on the tensor cores); 2: every call stays on the integer pipes."""
+    prev = B.set_conv_variant(request.param)
+    yield request.param
+    B.set_conv_variant(prev)
+
+
 def conv_inputs(case):
     N, C, H, W, O, kh, kw, stride, pad, pv = case
     rng = np.random.default_rng(abs(hash(case)) % (2**32))
@@ -166,7 +179,7 @@ def test_bconv2d_matches_oracle(B, oracle_mod, case, variant):
 
 
 @pytest.mark.parametrize("case", CONV_CASES)
-def test_fused_bn_sign_pack_matches_oracle(B, oracle_mod, case):
+def test_fused_bn_sign_pack_matches_oracle(B, oracle_mod, conv_variant, case):
     N, C, H, W, O, kh, kw, stride, pad, pv = case
     x, w = conv_inputs(case)
     o = oracle_mod
@@ -186,8 +199,9 @@ def test_fused_bn_sign_pack_matches_oracle(B, oracle_mod, case):
     assert 0 < np.count_nonzero(got) < got.size * 64 or O < 4
 
 
-@pytest.mark.parametrize("case", [CONV_CASES[0], CONV_CASES[3], CONV_CASES[4], CONV_CASES[8], CONV_CASES[12]])
-def test_bireal_block_epilogue_matches_oracle(B, oracle_mod, case):
+@pytest.mark.parametrize("case", [CONV_CASES[0], CONV_CASES[3], CONV_CASES[4], CONV_CASES[8], CONV_CASES[12],
+                                  CONV_CASES[13], CONV_CASES[14]])
+def test_bireal_block_epilogue_matches_oracle(B, oracle_mod, conv_variant, case):
     N, C, H, W, O, kh, kw, stride, pad, pv = case
     x, w = conv_inputs(case)
     o = oracle_mod
@@ -261,7 +275,7 @@ FULL = [(64, C, HW, C, 3, 1) for C, HW in synth.SWEEP_SHAPES] + [(256, 256, 28, 
 
 
 @pytest.mark.parametrize("cfg", FULL)
-def test_full_size_configs_on_sampled_outputs(B, oracle_mod, cfg):
+def test_full_size_configs_on_sampled_outputs(B, oracle_mod, conv_variant, cfg):
     N, C, HW, O, k, pad = cfg
     x, w = synth.conv_case(2 if N == 64 else 5, N, C, HW, HW, O, k, k, salt=C)
     a, wp = B.pack(dev(x)), B.pack_weights(dev(w))
@@ -284,8 +298,11 @@ def test_full_size_configs_on_sampled_outputs(B, oracle_mod, cfg):
     del g
     # and the whole packed output of the fused BN + sign + pack epilogue
     scale, shift = full_size_bn(C, N, O, K)
+    n0 = B.tc_launches()
     bits = B.bconv2d_bn_sign_pack(a, C, wp, dev(scale), dev(shift), (1, 1), (pad, pad), -1)
+    assert B.tc_launches() - n0 == (1 if conv_variant == 0 else 0)
     assert np.array_equal(u64(bits), oracle_mod.bn_sign_pack(full, scale, shift))
+    assert B.last_device_flag() == 0
 
 
 def test_full_size_pack_config(B, oracle_mod):

@@ -88,7 +88,10 @@ def test_tc_conv_and_epilogues_match_oracle(B, oracle_mod, case):
     got_nchw = B.tc_bconv2d(a, wt, st, (pad, pad), pv, B.NCHW).cpu().numpy()
     assert np.array_equal(got_nchw, np.transpose(acc, (0, 3, 1, 2)))
     # the xor/popcount kernel gives the same integers
+    prev, n0 = B.set_conv_variant(2), B.tc_launches()
     assert np.array_equal(B.bconv2d(a, C, wp, st, (pad, pad), pv, B.NHWC).cpu().numpy(), acc)
+    assert B.tc_launches() == n0
+    B.set_conv_variant(prev)
     # fused BN + sign + pack
     rng = np.random.default_rng(O)
     gamma, beta, mean, var = synth.bn_params(rng, O)
@@ -158,7 +161,11 @@ def test_tc_bgemm_matches_eq1(B, oracle_mod, shape):
     got = B.tc_bgemm(A, B.TcWeights(Bp, K), K).cpu().numpy()
     counts = oracle_mod.bgemm_xnor(u64(A), u64(Bp).reshape(N, -1), K)  # Eq. 1 as printed: agreeing positions
     assert np.array_equal(got, 2 * counts - K)
-    assert np.array_equal(got, B.bgemm(A, Bp.reshape(N, -1), K).cpu().numpy())
+    prev, n0 = B.set_conv_variant(2), B.tc_launches()
+    assert np.array_equal(got, B.bgemm(A, Bp.reshape(N, -1), K).cpu().numpy())  # the integer pipes
+    assert B.tc_launches() == n0
+    B.set_conv_variant(prev)
+    assert np.array_equal(got, B.bgemm(A, Bp.reshape(N, -1), K).cpu().numpy())  # either engine
 
 
 def test_tc_declines_what_it_does_not_cover(B):
@@ -424,7 +431,7 @@ def test_residual_ring_depths_in_a_child_process(ring):
     assert r.returncode == 0 and "ring ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
 
 
-# Packed-weight calls large enough for the route onto this engine (their CTAs expand the packed rows themselves): an odd
+# Packed-weight calls whose sign words (at least) run on this engine; its CTAs expand the packed rows themselves: an odd
 # last word of a cut channel tile (O and K odd), a channel tail, no 3x3 thirds, CTA pairs with a cut tile, the rows staged
 # behind the first activation buffer or (stride 2) in the only one, channels in groups, several resident tiles, odd rows out.
 BITS_ROUTE_CASES = [
@@ -457,8 +464,19 @@ def test_packed_weight_calls_on_this_engine_match_oracle(B, oracle_mod, case):
     y, want_ybits = o.bn_add_sign_pack(acc, scale, shift, res)
     want_bits = o.bn_sign_pack(acc, scale, shift)
     a, wp = B.pack(dev(x)), B.pack_weights(dev(w))
+    # every output form of this engine, whatever a packed-weight call would choose (the same kernels read the caller's rows)
+    wt, n0 = B.TcWeights(wp, C), B.tc_launches()
+    assert np.array_equal(B.tc_bconv2d(a, wt, st, (pad, pad), pv).cpu().numpy(), acc)
+    assert np.array_equal(u64(B.tc_bconv2d_bn_sign_pack(a, wt, dev(scale), dev(shift), st, (pad, pad), pv)), want_bits)
+    got_y, got_ybits = B.tc_bconv2d_bn_add_sign_pack(a, wt, dev(scale), dev(shift), dev(res), st, (pad, pad), pv)
+    assert np.array_equal(got_y.cpu().numpy().view(np.uint32), y.view(np.uint32))
+    assert np.array_equal(u64(got_ybits), want_ybits)
+    assert B.tc_launches() - n0 == 3
     off = torch.cat([wp.flatten()[:1], wp.flatten()])[1:].view(wp.shape)  # 8 bytes off a 16-byte boundary: the other engine
     for weights in (wp, off):
+        n0 = B.tc_launches()
+        B.bconv2d_bn_sign_pack(a, C, weights, dev(scale), dev(shift), st, (pad, pad), pv)
+        assert B.tc_launches() - n0 == (1 if weights is wp else 0)
         assert np.array_equal(B.bconv2d(a, C, weights, st, (pad, pad), pv).cpu().numpy(), acc)
         nchw = B.bconv2d(a, C, weights, st, (pad, pad), pv, out_layout=B.NCHW)
         assert np.array_equal(nchw.cpu().numpy(), acc.transpose(0, 3, 1, 2))
