@@ -318,6 +318,17 @@ __global__ void pack_weights_kernel(const float* __restrict__ w, int O, int C, i
 
 using namespace dabnn;
 
+// NHWC rows of no whole words: one contiguous run per CTA (pack_nhwc_flat) or one thread per word (pack_generic), which reads each
+// lane's row on its own.  The latter stays ahead where a row is short (17 channels, 200704 pixels: 4.27 against 5.44 us) and the pixels
+// many (38 channels, 33504 pixels: 3.64 against 4.98) or few (40 channels, 25 pixels: 2.43 / 2.85; 600 pixels of 39 channels: 3.72 /
+// 2.98), and where 32 long rows are more than a CTA reads in the time (about 9 us) that 64 loads in a row take, unless there are
+// enough such CTAs for their rate to count (1427 channels, 125 pixels: 9.1 / 17.7; 997 channels, 3248 pixels: 15.6 / 12.3).
+bool nhwc_flat_pays(long long npix, int C) {
+  if (C <= 32) return false;
+  if (C <= 48) return npix >= 256 && npix < 16384;
+  return (npix < 32 ? npix : 32) * C <= 18000 || npix >= 64 * 32;
+}
+
 template <typename T>
 dabnn_status pack_any(const T* x, dabnn_layout in_layout, dabnn_shape s, uint64_t* packed, void* stream,
                       dabnn_packed_layout pl = DABNN_PACKED_NHWC) {
@@ -351,10 +362,9 @@ dabnn_status pack_any(const T* x, dabnn_layout in_layout, dabnn_shape s, uint64_
     const long long cap = (long long)sm_count() * 16;
     if (blocks > cap) blocks = cap;
     pack_nhwc_c64<T><<<(unsigned)blocks, 256, 0, st>>>(x, total_words, packed);
-  } else if (!c2 && in_layout == DABNN_NHWC && s.C > 32 && s.C <= 4096 && aligned(x, 16)) {
-    // about 8192 values per CTA, 2048 where that leaves less than two CTAs per SM.  37 x 27 x 29 x 100: 7.16 -> 5.15 us, 200 x 14 x 14 x 300 23.3 -> 13.7,
-    // against one thread per word, which reads each lane's row on its own and stays ahead where a row is short (64 x 56 x 56
-    // x 17: 4.27 against 5.44)
+  } else if (!c2 && in_layout == DABNN_NHWC && s.C <= 4096 && aligned(x, 16) && nhwc_flat_pays((long long)s.N * HW, s.C)) {
+    // about 8192 values per CTA, 2048 where that leaves less than two CTAs per SM.  37 x 27 x 29 x 100: 7.16 -> 5.15 us, 200 x 14 x 14 x 300 23.3 -> 13.7
+    // against one thread per word
     const long long npix = (long long)s.N * HW;
     const int target = npix * s.C >= 2LL * 8192 * sm_count() ? 8192 : 2048;
     const int P = target / s.C >= 64 ? target / s.C / 32 * 32 : 32;

@@ -61,10 +61,12 @@ def test_pack_nchw(B, oracle_mod, shape):
     assert np.array_equal(got, oracle_mod.pack(x, oracle_mod.NCHW))
 
 
-# whole words of 64; one thread per word (few channels, one beyond the largest of the flat path); the flat-bitmap path: last
-# vectors of one, two and three values, several pixel tiles, large tiles, its largest C
+# whole words of 64; one thread per word and the flat-bitmap path on both sides of every line between them: few channels, short
+# rows with few and many pixels, long rows with few pixels; last vectors of one, two and three values, several pixel tiles,
+# large tiles, the largest C of the path and one beyond it
 PACK_NHWC_SHAPES = [(2, 14, 14, 64), (3, 9, 7, 256), (2, 5, 5, 70), (1, 3, 3, 4), (4, 31, 17, 128), (1, 1, 1, 1), (3, 1, 1, 1),
-                    (1, 7, 11, 35), (1, 7, 9, 35), (2, 33, 17, 33), (37, 27, 29, 100), (90, 28, 28, 70), (1, 6, 6, 4090), (1, 3, 3, 4099)]
+                    (1, 7, 11, 35), (17, 7, 9, 35), (2, 33, 17, 33), (37, 27, 29, 100), (90, 28, 28, 70), (3, 5, 7, 61), (1, 7, 9, 53), (1, 6, 6, 4090),
+                    (1, 1, 4, 4090), (1, 2050, 1, 4090), (1, 3, 3, 4099), (1, 5, 25, 1427), (1, 3, 7, 45), (6, 52, 53, 38)]
 
 
 @pytest.mark.parametrize("shape", PACK_NHWC_SHAPES)
