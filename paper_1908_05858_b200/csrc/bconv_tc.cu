@@ -227,9 +227,9 @@ __device__ __forceinline__ void st_global_v8(void* p, uint32_t a, uint32_t b, ui
                "r"(f), "r"(g2), "r"(h)
                : "memory");
 }
-// The same with an evict-first policy in L2 (made once per thread): for output that nothing in this library reads back (the
-// int32 sums), so that it drains to DRAM as it is produced instead of displacing the weights and activations that the
-// next launches read.
+// The same with an evict-first policy in L2 (made once per thread): for the int32 sums, as the integer-pipe kernel's streaming
+// stores, so that they drain to DRAM as they are produced instead of displacing the weights and activations that the next
+// launches read.  (A dabnn_pack_i32 of them is the exception: it finds of a large tensor what has not drained yet.)
 __device__ __forceinline__ uint64_t evict_first_policy() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
@@ -933,7 +933,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       // every later chunk one chunk ahead of its use.
       float rpre[32];
       auto load_res = [&](int c0) {
-        if (EPI == EPI_BIREAL && wide_y && my_valid && !tma_res) {
+        if (!tma_res && EPI == EPI_BIREAL && wide_y && my_valid) {
           const int o = nt * NT + c0;
           const int nch = min(32, g.O - o);
           const float* rs = g.residual + (long long)my_m * g.O + o;
@@ -1013,8 +1013,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
           continue;
         }
         float rc[32];
-        if (false) {
-        } else if (EPI == EPI_BIREAL) {
+        if (EPI == EPI_BIREAL) {
 #pragma unroll
           for (int j = 0; j < 32; j++) rc[j] = rpre[j];
           if (c0 + c_step < NT) load_res(c0 + c_step);

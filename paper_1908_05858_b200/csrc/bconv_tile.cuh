@@ -339,8 +339,8 @@ __device__ __forceinline__ void bconv_tile(const BConvArgs& g, const long long b
         v[j] = g.Kbits - 2 * cnt;
       }
       const int o = o0 + wrow0;
-      // (streaming stores: the int32 sums are read by nothing in this library, and kept out of the way in L2 they do
-      // not displace the weights and activations that the following launches read)
+      // (streaming stores: only dabnn_pack_i32 reads the int32 sums back, and kept out of the way in L2 they do not displace
+      // the weights and activations that the following launches read)
       if (!g.out_nchw) {
         int32_t* dst = g.out + m * g.O + o;
         if (TO % 4 == 0 && o + TO <= g.O && (g.O & 3) == 0 && (reinterpret_cast<uintptr_t>(g.out) & 15) == 0) {
