@@ -82,7 +82,8 @@ dabnn_status dabnn_pack_i32(const int32_t* x, dabnn_layout in_layout, dabnn_shap
  *   dabnn_packed_words   64-bit words of a packed tensor in either layout (0 for an invalid shape or layout)
  *   dabnn_pack_as        dabnn_pack into the chosen layout (packed: 16-byte aligned for NC1HWC2)
  *   dabnn_bconv2d_from   dabnn_bconv2d reading activations in the chosen layout (weights stay [O][kh][kw][Cw]); the
- *                        integers are the same whichever layout the activations are in. */
+ *                        integers are the same whichever layout the activations are in.  Always on the integer pipes, so
+ *                        that the two layouts are compared on one engine. */
 typedef enum { DABNN_PACKED_NHWC = 0, DABNN_PACKED_NC1HWC2 = 1 } dabnn_packed_layout;
 size_t dabnn_packed_words(dabnn_shape s, dabnn_packed_layout packed_layout);
 dabnn_status dabnn_pack_as(const float* x, dabnn_layout in_layout, dabnn_shape s, dabnn_packed_layout packed_layout,
@@ -284,7 +285,7 @@ dabnn_status dabnn_tc_bconv2d_bn_add_sign_pack(const uint64_t* a_packed, dabnn_s
                                                dabnn_conv cv, const float* scale, const float* shift, const float* residual,
                                                float* y_out, uint64_t* out_packed, void* stream);
 /* Eq. 1 (BGEMM) on the tensor-core engine: dabnn_bgemm with B prepared once by
- * dabnn_tc_prepare_weights(B, N, Kbits, 1, 1, b_tc) (dabnn_tc_weights_bytes(N, Kbits, 1, 1) bytes; Kbits <= 512).  Same integers. */
+ * dabnn_tc_prepare_weights(B, N, Kbits, 1, 1, b_tc) (dabnn_tc_weights_bytes(N, Kbits, 1, 1) bytes; Kbits <= 9216).  Same integers. */
 dabnn_status dabnn_tc_bgemm(const uint64_t* A, int M, const void* b_tc, int N, int Kbits, int32_t* C, void* stream);
 unsigned long long dabnn_tc_launches(void);
 int dabnn_tc_error_flag(void);
