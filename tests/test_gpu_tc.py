@@ -347,6 +347,29 @@ def test_a_wait_that_runs_out_sets_the_flag_and_leaves_the_device_usable(B, orac
         B.tc_wait_expiry_selftest(a, wt, (1, 1), (pad, pad), -1, wait_polls=1 << 20)  # limit beyond a few milliseconds: refused
 
 
+@pytest.mark.parametrize("N,C,H,O,k,stride", [
+    (60, 64, 28, 64, 1, 1),      # 1x1: a handful of MMAs between two waits
+    (30, 1024, 10, 64, 1, 1),    # channel groups: several activation buffers per tile
+    (20, 256, 14, 128, 3, 2),    # stride 2, weights ready a row of taps at a time
+    (40, 256, 14, 256, 3, 1),    # pairs where the launch is large enough, several channel tiles per CTA
+])
+def test_waits_that_run_out_part_no_lanes(B, oracle_mod, N, C, H, O, k, stride):
+    """Limits from one poll on, at which the lanes of a warp need not agree whether a barrier had completed: each launch comes back
+    by itself, and the ordinary launch behind it gives the oracle's integers."""
+    o = oracle_mod
+    rng = np.random.default_rng(C + k)
+    x, w = rng.standard_normal((N, C, H, H)).astype(np.float32), rng.standard_normal((O, C, k, k)).astype(np.float32)
+    geom = ((stride, stride), (k // 2, k // 2), -1)
+    want = o.bconv_bits(o.pack(x), C, o.pack_weights(w), *geom, o.NHWC)
+    a, wt = B.pack(dev(x)), B.TcWeights(B.pack_weights(dev(w)), C)
+    for polls in (1, 2, 3, 4, 6, 10, 30, 300):
+        for _ in range(4):
+            B.tc_wait_expiry_selftest(a, wt, *geom, wait_polls=polls)
+        assert B.stream_status() == B.ERR_TIMEOUT
+        assert np.array_equal(B.tc_bconv2d(a, wt, *geom, B.NHWC).cpu().numpy(), want)
+        assert B.stream_status() == 0
+
+
 def tc_matrix_cases():
     """Channel words 1..8 x filter sizes 1, 2, 3, 4, 5, 7 x strides 1, 2: every count of K blocks per tap through the
     unrolled 3x3 issue path and the runtime tap loops of the other filters, at a size with several tiles and a ragged

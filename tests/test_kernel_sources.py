@@ -1,0 +1,30 @@
+"""Rules that the kernels keep and that no run without a fault can show: checked in their source."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1908_05858_b200", "csrc")
+
+
+def source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def test_bounded_waits_are_answered_by_the_warp():
+    """Every role of the tensor-core kernel runs warp-wide instructions behind its waits, so a wait that runs out, or a failure of
+    another role, has to part no lanes: each wait's result goes through a vote, and the failure flag is read through one or once all
+    roles have met."""
+    text = source("bconv_tc.cu")
+    warp_wait = text[text.index("bool mbar_wait_warp("):]
+    warp_wait = warp_wait[:warp_wait.index("\n}")]
+    assert "if (__all_sync(0xFFFFFFFFu, done != 0)) return true;" in warp_wait and "__any_sync(0xFFFFFFFFu, *fail != 0)" in warp_wait
+    kernel = text[text.index("bconv_tc_kernel("):text.index("tc_prepare_weights_kernel")]
+    assert "mbar_wait_warp<PAIR>(" in kernel  # the role that issues the MMAs
+    calls = [m.start() for m in re.finditer(r"\bmbar_wait\w*\(", kernel)]
+    assert len(calls) >= 5
+    for at in calls:
+        vote = kernel.rfind("__all_sync(0xFFFFFFFFu", 0, at)
+        assert vote >= 0 and ";" not in kernel[vote:at], kernel[max(0, at - 200):at + 100]
+    for m in re.finditer(r"\*s_fail != 0", kernel):
+        line = kernel[kernel.rfind("\n", 0, m.start()) + 1:kernel.index("\n", m.end())]
+        assert "__any_sync(0xFFFFFFFFu, *s_fail != 0)" in line or "*s_fail != 0 && tid == 0" in line, line
