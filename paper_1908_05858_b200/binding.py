@@ -37,6 +37,10 @@ EXPORTS = (
     "dabnn_bireal18_forward_stem_module", "dabnn_tc_bgemm", "dabnn_tc_launches",
 )
 
+# what the extension module calls, in its order
+_NATIVE_ENTRIES = ("dabnn_pack", "dabnn_bconv2d", "dabnn_bconv2d_bn_sign_pack", "dabnn_bconv2d_bn_add_sign_pack", "dabnn_tc_bconv2d",
+                   "dabnn_tc_bconv2d_bn_sign_pack", "dabnn_tc_bconv2d_bn_add_sign_pack")
+
 PACKED_NHWC = 0
 PACKED_NC1HWC2 = 1
 
@@ -148,9 +152,7 @@ def lib() -> ctypes.CDLL:
             getattr(L, name).restype = ci
         from . import _native as native
 
-        native.bind(*[ctypes.cast(getattr(L, name), vp).value for name in (
-            "dabnn_pack", "dabnn_bconv2d", "dabnn_bconv2d_bn_sign_pack", "dabnn_bconv2d_bn_add_sign_pack", "dabnn_tc_bconv2d",
-            "dabnn_tc_bconv2d_bn_sign_pack", "dabnn_tc_bconv2d_bn_add_sign_pack")])
+        native.bind(*[ctypes.cast(getattr(L, name), vp).value for name in _NATIVE_ENTRIES], _check)
         _native, _lib = native, L
     return _lib
 

@@ -3,8 +3,9 @@
 // calls took 18.1 us of host time, most of it attribute look-ups, struct marshalling and torch.empty's argument parser; 8.4 like this.
 //
 // Only the ordinary case is handled here -- plain contiguous CUDA tensors of the right types on the current device, outputs made
-// by torch.  Everything else, errors included, returns None: binding.py then takes its general path, which converts, allocates
-// through the caller's hook, or raises.  Nothing is kept from one call for the next.
+// by torch.  Everything else, refused arguments included, returns None: binding.py then takes its general path, which converts,
+// allocates through the caller's hook, or raises.  A launch that failed is not made again: its status is raised from here.  Nothing
+// is kept from one call for the next.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -28,11 +29,12 @@ struct Entries {
   decltype(&dabnn_tc_bconv2d_bn_add_sign_pack) tc_bn_add_sign_pack;
 };
 Entries g_entries;
+PyObject* g_check;  // binding.py's: raises what a status stands for
 
 PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
   static_assert(sizeof(Entries) == 7 * sizeof(void*), "one address per entry");
-  if (n != 7) {
-    PyErr_SetString(PyExc_TypeError, "bind takes seven addresses");
+  if (n != 8 || !PyCallable_Check(args[7])) {
+    PyErr_SetString(PyExc_TypeError, "bind takes seven addresses and what raises a status");
     return nullptr;
   }
   void* address[7];
@@ -41,6 +43,7 @@ PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (PyErr_Occurred()) return nullptr;
   }
   memcpy(&g_entries, address, sizeof(g_entries));
+  Py_XSETREF(g_check, Py_NewRef(args[7]));
   Py_RETURN_NONE;
 }
 
@@ -76,14 +79,35 @@ at::Tensor make(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& li
   return at::empty(sizes, at::TensorOptions().dtype(type).device(like.device()));
 }
 
-// The call itself, with the interpreter released as ctypes does; any status but OK goes to the general path, which reports it.
+// The call itself, with the interpreter released as ctypes does.
 template <typename F>
-bool done(F f) {
+dabnn_status status_of(F f) {
   dabnn_status s;
   Py_BEGIN_ALLOW_THREADS
   s = f();
   Py_END_ALLOW_THREADS
-  return s == DABNN_OK;
+  return s;
+}
+
+// What a call with a status other than OK returns.  Arguments are refused before anything is launched: the general path meets the
+// same refusal and reports it.  After any other status the launch may have gone out, and the library has read (and so cleared) the
+// runtime's error: a second call could succeed in silence.
+PyObject* not_made(dabnn_status s) {
+  switch (s) {
+    case DABNN_ERR_NULL:
+    case DABNN_ERR_SHAPE:
+    case DABNN_ERR_UNSUPPORTED:
+    case DABNN_ERR_ALIGNMENT:
+    case DABNN_ERR_WORKSPACE:
+    case DABNN_ERR_STATIC_LIMIT: Py_RETURN_NONE;
+    default: break;
+  }
+  PyObject* returned = PyObject_CallFunction(g_check, "i", (int)s);
+  if (returned != nullptr) {
+    Py_DECREF(returned);
+    PyErr_Format(PyExc_RuntimeError, "dabnn status %d", (int)s);
+  }
+  return nullptr;
 }
 
 template <typename F>
@@ -164,7 +188,8 @@ PyObject* pack(PyObject*, PyObject* const* args, Py_ssize_t n) {
     at::Tensor out = make({in.N, in.H, in.W, (in.C + 63LL) / 64}, at::kLong, *x);
     const float* src = static_cast<const float*>(x->data_ptr());
     uint64_t* dst = static_cast<uint64_t*>(out.data_ptr());
-    if (!done([&] { return g_entries.pack(src, (dabnn_layout)layout, in, dst, stream.stream()); })) Py_RETURN_NONE;
+    const dabnn_status s = status_of([&] { return g_entries.pack(src, (dabnn_layout)layout, in, dst, stream.stream()); });
+    if (s != DABNN_OK) return not_made(s);
     return THPVariable_Wrap(std::move(out));
   });
 }
@@ -179,11 +204,11 @@ PyObject* conv_int32(decltype(&dabnn_tc_bconv2d) entry, decltype(&dabnn_bconv2d)
     at::Tensor out = sums_like(g, layout);
     const uint64_t* ap = static_cast<const uint64_t*>(g.a->data_ptr());
     int32_t* dst = static_cast<int32_t*>(out.data_ptr());
-    const bool ok = done([&] {
+    const dabnn_status s = status_of([&] {
       return entry != nullptr ? entry(ap, g.in, g.w, g.O, g.cv, dst, (dabnn_layout)layout, g.stream)
                               : packed_entry(ap, g.in, static_cast<const uint64_t*>(g.w), g.O, g.cv, dst, (dabnn_layout)layout, g.stream);
     });
-    if (!ok) Py_RETURN_NONE;
+    if (s != DABNN_OK) return not_made(s);
     return THPVariable_Wrap(std::move(out));
   });
 }
@@ -206,11 +231,11 @@ PyObject* conv_signs(decltype(&dabnn_tc_bconv2d_bn_sign_pack) entry, decltype(&d
     at::Tensor out = words_like(g);
     const uint64_t* ap = static_cast<const uint64_t*>(g.a->data_ptr());
     uint64_t* dst = static_cast<uint64_t*>(out.data_ptr());
-    const bool ok = done([&] {
+    const dabnn_status s = status_of([&] {
       return entry != nullptr ? entry(ap, g.in, g.w, g.O, g.cv, scale, shift, dst, g.stream)
                               : packed_entry(ap, g.in, static_cast<const uint64_t*>(g.w), g.O, g.cv, scale, shift, dst, g.stream);
     });
-    if (!ok) Py_RETURN_NONE;
+    if (s != DABNN_OK) return not_made(s);
     return THPVariable_Wrap(std::move(out));
   });
 }
@@ -233,11 +258,11 @@ PyObject* conv_block(decltype(&dabnn_tc_bconv2d_bn_add_sign_pack) entry, decltyp
     const float* rp = static_cast<const float*>(residual->data_ptr());
     float* yp = static_cast<float*>(y.data_ptr());
     uint64_t* bp = bits.defined() ? static_cast<uint64_t*>(bits.data_ptr()) : nullptr;
-    const bool ok = done([&] {
+    const dabnn_status s = status_of([&] {
       return entry != nullptr ? entry(ap, g.in, g.w, g.O, g.cv, scale, shift, rp, yp, bp, g.stream)
                               : packed_entry(ap, g.in, static_cast<const uint64_t*>(g.w), g.O, g.cv, scale, shift, rp, yp, bp, g.stream);
     });
-    if (!ok) Py_RETURN_NONE;
+    if (s != DABNN_OK) return not_made(s);
     PyObject* py = THPVariable_Wrap(std::move(y));
     if (py == nullptr) return nullptr;
     PyObject* pb = bits.defined() ? THPVariable_Wrap(std::move(bits)) : Py_NewRef(Py_None);

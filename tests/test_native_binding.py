@@ -1,4 +1,5 @@
 """The extension module's calls give what the ctypes path gives, and leave to that path whatever is not an ordinary call."""
+import ctypes
 import threading
 
 import pytest
@@ -116,3 +117,32 @@ def test_what_was_refused_stays_refused(native):
                 path(f)
             seen.append((e.type, str(e.value)))
         assert seen[0] == seen[1]
+
+
+@pytest.mark.gpu
+def test_a_launch_that_failed_is_reported_and_not_made_again(native):
+    """The library reads and clears the runtime's last error, so a second call after a failed one could succeed in silence.  With
+    entries that only return a status: a failed launch raises, refused arguments go to the general path."""
+    x, res, v = torch.randn(2, 64, 6, 6, device="cuda"), torch.randn(2, 6, 6, 8, device="cuda"), torch.ones(8, device="cuda")
+    a, w = plain(lambda: B.pack(x)), plain(lambda: B.pack_weights(torch.randn(8, 64, 3, 3, device="cuda")))
+    wt, geom = B.TcWeights(w, 64), ((1, 1), (1, 1), -1)
+    calls = [lambda: B.pack(x), lambda: B.bconv2d(a, 64, w, *geom), lambda: B.bconv2d_bn_sign_pack(a, 64, w, v, v, *geom),
+             lambda: B.bconv2d_bn_add_sign_pack(a, 64, w, v, v, res, *geom), lambda: B.tc_bconv2d(a, wt, *geom),
+             lambda: B.tc_bconv2d_bn_sign_pack(a, wt, v, v, *geom), lambda: B.tc_bconv2d_bn_add_sign_pack(a, wt, v, v, res, *geom)]
+    want = [general(f) for f in calls]
+    made, status = [], [0]
+    fake = ctypes.CFUNCTYPE(ctypes.c_int)(lambda: made.append(1) or status[0])
+    try:
+        native.bind(*[ctypes.cast(fake, ctypes.c_void_p).value] * len(B._NATIVE_ENTRIES), B._check)
+        for f, y in zip(calls, want, strict=True):
+            for status[0] in (6, 7):  # DABNN_ERR_CUDA, DABNN_ERR_TIMEOUT
+                made.clear()
+                with pytest.raises(B.DabnnError, match="dabnn status %d" % status[0]):
+                    plain(f)
+                assert len(made) == 1
+            status[0] = 2  # DABNN_ERR_SHAPE
+            got = plain(f)
+            assert all(torch.equal(p, q) for p, q in zip(*(t if isinstance(t, tuple) else (t,) for t in (got, y)), strict=True))
+    finally:
+        native.bind(*[ctypes.cast(getattr(B.lib(), name), ctypes.c_void_p).value for name in B._NATIVE_ENTRIES], B._check)
+    assert torch.equal(plain(calls[0]), want[0])
