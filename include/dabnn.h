@@ -65,7 +65,7 @@ const char* dabnn_status_string(dabnn_status s);
 
 /* ceil(C/64): 64-bit words per pixel (or per weight tap). */
 size_t dabnn_words_per_pixel(int C);
-/* floor((in + 2*pad - k)/stride) + 1 (may be <= 0: no output). */
+/* floor((in + 2*pad - k)/stride) + 1; 0: no output, or a padded size that no int holds. */
 int dabnn_out_dim(int in, int k, int stride, int pad);
 
 /* Section 2.1.1 -- binarize + pack activations.

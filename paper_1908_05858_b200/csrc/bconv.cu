@@ -16,6 +16,7 @@
 // bit_mac -- and popcounts only the carry word: half the POPCs, so the bound doubles to 32 word
 // pairs/clk/SM (XU full, ALU at 3/4), and the accumulation is an IMAD on the FMA pipe.
 // Both give sum popcount(a xor w) exactly.
+#include <limits.h>
 #include <stdlib.h>
 
 #include "common.cuh"
@@ -238,10 +239,9 @@ extern "C" int dabnn_set_conv_tile(int tile) {
 extern "C" size_t dabnn_words_per_pixel(int C) { return C <= 0 ? 0 : (size_t)((C + 63) / 64); }
 
 extern "C" int dabnn_out_dim(int in, int k, int stride, int pad) {
-  if (stride <= 0) return 0;
-  const int span = in + 2 * pad - k;
-  if (span < 0) return 0;
-  return span / stride + 1;
+  const long long padded = (long long)in + 2LL * pad, span = padded - k;
+  if (stride <= 0 || span < 0 || padded > INT_MAX || span / stride >= INT_MAX) return 0;
+  return (int)(span / stride + 1);
 }
 
 extern "C" const char* dabnn_status_string(dabnn_status s) {

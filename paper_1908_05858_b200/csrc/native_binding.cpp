@@ -70,8 +70,10 @@ bool pair(PyObject* o, int& a, int& b) {
   return PyTuple_CheckExact(o) && PyTuple_GET_SIZE(o) == 2 && integer(PyTuple_GET_ITEM(o, 0), a) && integer(PyTuple_GET_ITEM(o, 1), b);
 }
 
+// dabnn_out_dim; -1 for a padded size that no int holds.
 int out_dim(int in, int k, int stride, int pad) {
-  const long long span = (long long)in + 2LL * pad - k;
+  const long long padded = (long long)in + 2LL * pad, span = padded - k;
+  if (padded > INT_MAX) return -1;
   return span >= 0 && stride > 0 ? (int)(span / stride + 1) : 0;
 }
 
@@ -142,6 +144,7 @@ bool geometry(Geometry& g, PyObject* a, PyObject* stride, PyObject* pad, PyObjec
   if (g.cv.stride_h <= 0 || g.cv.stride_w <= 0 || !fits(g.cv.pad_h) || !fits(g.cv.pad_w)) return false;
   g.OH = out_dim(g.in.H, g.cv.kh, g.cv.stride_h, g.cv.pad_h);
   g.OW = out_dim(g.in.W, g.cv.kw, g.cv.stride_w, g.cv.pad_w);
+  if (g.OH < 0 || g.OW < 0) return false;
   const auto stream = c10::cuda::getCurrentCUDAStream();
   g.stream = stream.stream();
   return g.a->device() == stream.device();

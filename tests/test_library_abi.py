@@ -39,6 +39,9 @@ def test_helpers(L):
     assert L.dabnn_words_per_pixel(0) == 0
     assert L.dabnn_out_dim(56, 3, 1, 1) == 56 and L.dabnn_out_dim(56, 3, 2, 1) == 28 and L.dabnn_out_dim(7, 3, 2, 1) == 4
     assert L.dabnn_out_dim(2, 5, 1, 0) == 0
+    big = 2**31 - 1  # 2 * pad passes through 2^32 - 2: 10 rows, if the sum is taken modulo 2^32
+    assert L.dabnn_out_dim(14, 3, 1, big) == 0 and L.dabnn_out_dim(14, 3, 2**30, big) == 0 and L.dabnn_out_dim(14, 3, 1, 2**30) == 0
+    assert L.dabnn_out_dim(13, 1, 1, 2**30 - 7) == big and L.dabnn_out_dim(big, 1, 1, 0) == big and L.dabnn_out_dim(big, big, 1, 0) == 1
     assert L.dabnn_status_string(0) == b"ok"
     assert b"workspace" in L.dabnn_status_string(5)
     assert L.dabnn_bireal18_workspace_bytes(0) == 0
@@ -63,6 +66,11 @@ def test_argument_errors_are_reported_before_any_launch(L):
     assert L.dabnn_bconv2d(fake, s, fake, 8, Conv(3, 3, 1, 1, 1, 1, 0), fake, 1, None) == 2   # pad_value not +-1
     assert L.dabnn_bconv2d(fake, s, fake, 8, Conv(3, 3, 0, 1, 1, 1, -1), fake, 1, None) == 2  # stride 0
     assert L.dabnn_bconv2d(fake, s, fake, 8, Conv(7, 7, 1, 1, 0, 0, -1), fake, 1, None) == 2  # empty output
+    for pad in (2**31 - 1, 2**30):                                                             # a padded size beyond an int
+        wide = Conv(3, 3, 1, 1, pad, pad, -1)
+        assert L.dabnn_bconv2d(fake, Shape(1, 64, 14, 14), fake, 8, wide, fake, 1, None) == 2
+        assert L.dabnn_tc_bconv2d(fake, Shape(1, 64, 14, 14), fake, 8, wide, fake, 1, None) == 2
+        assert L.dabnn_binary_layer_host_workspace_bytes(Shape(1, 64, 14, 14), 8, wide) == 0
     assert L.dabnn_bconv2d(odd, s, fake, 8, cv, fake, 1, None) == 4
     assert L.dabnn_bconv2d(fake, s, fake, 8, cv, fake, 5, None) == 2                           # bad layout
     assert L.dabnn_bconv2d_bn_sign_pack(fake, s, fake, 8, cv, None, fake, fake, None) == 1

@@ -105,9 +105,10 @@ def test_same_as_the_general_path(native, N, C, H, W, O, k, stride):
 def test_what_was_refused_stays_refused(native):
     x = torch.randn(2, 64, 6, 6, device="cuda")
     a, w = plain(lambda: B.pack(x)), plain(lambda: B.pack_weights(torch.randn(8, 64, 3, 3, device="cuda")))
-    v = torch.ones(8, device="cuda")
+    v, wt = torch.ones(8, device="cuda"), plain(lambda: B.TcWeights(w, 64))
     calls = [lambda: B.pack(x.double()), lambda: B.pack(x.half()), lambda: B.pack(x[0]), lambda: B.pack(x.cpu()), lambda: B.pack(x[:0]),
              lambda: B.bconv2d(a, 65, w), lambda: B.bconv2d(a, 64, w, (0, 1)), lambda: B.bconv2d(a, 64, w, (1, 1), (0, 0), 0),
+             lambda: B.bconv2d(a, 64, w, (1, 1), (2**31 - 1, 2**31 - 1)), lambda: B.tc_bconv2d(a, wt, (1, 1), (2**31 - 1, 2**31 - 1)),
              lambda: B.bconv2d(a, 64, w, (1, 1), (-1, 0)), lambda: B.bconv2d(a.int(), 64, w), lambda: B.bconv2d(a[:, :2, :2].contiguous(), 64, w),
              lambda: B.bconv2d_bn_sign_pack(a, 64, w, v.double(), v), lambda: B.bconv2d_bn_add_sign_pack(a, 64, w, v, v, torch.zeros(2, 4, 4, 7, device="cuda"))]
     for f in calls:
