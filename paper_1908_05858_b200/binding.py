@@ -1,8 +1,9 @@
 """Thin binding over the C ABI of ``libdabnn_b200.so`` (see ``include/dabnn.h``).
 
-The per-layer calls on ordinary tensors go through ``_native.so`` (csrc/native_binding.cpp), which does what the ctypes code
-below does without Python in between, and returns None for everything else: then, and for all other entry points, the ctypes code
-runs.  A pack and a small convolution, one after the other: 18.1 us of host time through ctypes, 8.4 through the module.
+The per-layer calls on ordinary tensors go through an extension module (csrc/native_binding.cpp), which does what the ctypes code
+below does without Python in between, and returns None for everything else: then, for all other entry points, and where the module
+has not been built for this interpreter and this torch, the ctypes code runs.  A pack and a small convolution, one after the other:
+18.1 us of host time through ctypes, 8.4 through the module.
 
 Argument marshalling only: every function checks dtypes / devices, allocates the output tensor with
 torch (torch owns device memory and the stream) and calls the entry point of the same name.  There
@@ -14,7 +15,10 @@ Packed tensors are ``torch.int64`` on the device (the bit pattern of the library
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import sysconfig
+import warnings
 from typing import Optional, Sequence
 
 import torch
@@ -24,7 +28,6 @@ NHWC = 1
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdabnn_b200.so")
-NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 EXPORTS = (
     "dabnn_status_string", "dabnn_words_per_pixel", "dabnn_out_dim", "dabnn_pack", "dabnn_pack_i32", "dabnn_pack_weights",
@@ -79,12 +82,32 @@ _lib: Optional[ctypes.CDLL] = None
 _native = None  # the extension module, once the library is loaded
 
 
+def native_path() -> str:
+    """The extension module's file.  It is compiled against one interpreter and one torch, so its name carries both: after a change
+    of either it counts as not built."""
+    return os.path.join(_HERE, "_native.torch-%s%s" % (torch.__version__, sysconfig.get_config_var("EXT_SUFFIX")))
+
+
+def _load_native(L: ctypes.CDLL):
+    """The extension module, bound to the library's entry points; None, with a warning, where it cannot be loaded."""
+    try:
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", native_path())
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+    except ImportError as e:
+        warnings.warn("per-layer calls go through ctypes, which takes about twice the host time: %s (run `python -m "
+                      "paper_1908_05858_b200.build` for the extension module)" % e, RuntimeWarning, stacklevel=3)
+        return None
+    native.bind(*[ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _NATIVE_ENTRIES], _check)
+    return native
+
+
 def lib() -> ctypes.CDLL:
     """Loads the CUDA library; raises if it has not been built (no fallback exists)."""
     global _lib, _native
     if _lib is None:
-        if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
-            raise DabnnError("libdabnn_b200.so or _native.so is missing: run `python -m paper_1908_05858_b200.build` "
+        if not os.path.exists(LIB_PATH):
+            raise DabnnError("libdabnn_b200.so is missing: run `python -m paper_1908_05858_b200.build` "
                              "(or __graft_entry__.build()) first; there is no CPU fallback")
         L = ctypes.CDLL(LIB_PATH)
         vp, ci = ctypes.c_void_p, ctypes.c_int
@@ -150,10 +173,7 @@ def lib() -> ctypes.CDLL:
         for name in ("dabnn_pack", "dabnn_pack_weights", "dabnn_bconv2d", "dabnn_bconv2d_bn_sign_pack",
                      "dabnn_bconv2d_bn_add_sign_pack", "dabnn_bn_fold", "dabnn_bireal18_forward"):
             getattr(L, name).restype = ci
-        from . import _native as native
-
-        native.bind(*[ctypes.cast(getattr(L, name), vp).value for name in _NATIVE_ENTRIES], _check)
-        _native, _lib = native, L
+        _native, _lib = _load_native(L), L
     return _lib
 
 

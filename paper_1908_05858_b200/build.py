@@ -1,7 +1,7 @@
-"""Builds libdabnn_b200.so (sm_100a only) from csrc/ with nvcc, in-tree, beside this file, and the Python extension _native.so."""
+"""Builds libdabnn_b200.so (sm_100a only) from csrc/ with nvcc, in-tree, beside this file, and the binding's Python
+extension for the interpreter and the torch that run this."""
 from __future__ import annotations
 
-import importlib.util
 import os
 import subprocess
 import sys
@@ -11,7 +11,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdabnn_b200.so")
-NATIVE = os.path.join(HERE, "_native.so")
 SOURCES = ["pack.cu", "bconv.cu", "bconv_tc.cu", "bireal18.cu", "stem_module.cu", "host_api.cu"]
 # -fmad=false: no implicit contraction of fp32 mul+add; every fused multiply-add is an explicit fmaf.
 NVCC_FLAGS = [
@@ -30,24 +29,34 @@ def _stale() -> bool:
 
 def build_native(force: bool = False) -> str:
     """The extension module: host code only, against torch's headers and libraries (which torch has loaded before it)."""
+    import torch
+
+    from .binding import native_path
+
+    native = native_path()
     src = os.path.join(CSRC, "native_binding.cpp")
     deps = [src, os.path.join(ROOT, "include", "dabnn.h"), __file__]
-    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
-        return NATIVE
-    torch_dir = list(importlib.util.find_spec("torch").submodule_search_locations)[0]
+    if not force and os.path.exists(native) and all(os.path.getmtime(d) <= os.path.getmtime(native) for d in deps):
+        return native
+    torch_dir = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    tmp = native + ".tmp.%d" % os.getpid()
     subprocess.check_call([
         os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"),
         "-isystem", os.path.join(torch_dir, "include"), "-isystem", os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
         "-isystem", os.path.join(cuda, "include"), "-isystem", sysconfig.get_paths()["include"], src, "-o", tmp,
         "-L", os.path.join(torch_dir, "lib"), "-lc10", "-ltorch_cpu", "-ltorch", "-ltorch_python", "-lc10_cuda"])
-    os.replace(tmp, NATIVE)
-    return NATIVE
+    os.replace(tmp, native)
+    return native
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    build_native(force)
+    lib = build_library(force, verbose)
+    build_native(force)  # (after the library, which needs none of torch's headers and can be used without it)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,5 +1,6 @@
 """The extension module's calls give what the ctypes path gives, and leave to that path whatever is not an ordinary call."""
 import ctypes
+import os
 import threading
 
 import pytest
@@ -26,6 +27,33 @@ def test_leaves_everything_but_cuda_tensors_alone(native):
         B.pack(x)
     with pytest.raises(TypeError):
         native.bind(1)
+
+
+def test_the_library_loads_without_the_module(native, monkeypatch, tmp_path):
+    """The module is a faster way to make the same calls: missing, or not loadable, it leaves them to ctypes."""
+    broken = tmp_path / os.path.basename(B.native_path())
+    broken.write_bytes(b"not a shared object")
+    for path in (str(tmp_path / ("absent" + broken.name)), str(broken)):
+        monkeypatch.setattr(B, "native_path", lambda: path)
+        monkeypatch.setattr(B, "_lib", None)
+        monkeypatch.setattr(B, "_native", native)
+        with pytest.warns(RuntimeWarning, match="ctypes"):
+            assert B.lib().dabnn_words_per_pixel(65) == 2
+        assert B._native is None
+        with pytest.raises(B.DabnnError):
+            B.pack(torch.zeros(1, 64, 4, 4))
+
+
+def test_the_module_of_another_torch_or_interpreter_is_not_taken(native, monkeypatch):
+    from paper_1908_05858_b200 import build
+
+    path = B.native_path()
+    assert os.path.exists(path) and build.build_native() == path
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".other")
+    assert not os.path.exists(B.native_path())
+    monkeypatch.undo()
+    monkeypatch.setattr(B.sysconfig, "get_config_var", lambda name: ".cpython-399.so")
+    assert not os.path.exists(B.native_path())
 
 
 def general(f):
