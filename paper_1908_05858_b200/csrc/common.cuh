@@ -68,7 +68,8 @@ inline bool chain_enabled() {
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The same for a pointer to what the previous kernel wrote: loads through the result cannot be moved above the wait, not even those
-// that count as invariant (__restrict__, __ldcs).
+// that count as invariant (__ldg, and any through a const __restrict__ pointer, whose cache hint keeps them in place only where the
+// intrinsic is a volatile asm).
 template <typename T>
 __device__ __forceinline__ const T* chain_wait_for(const T* p) {
   asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");

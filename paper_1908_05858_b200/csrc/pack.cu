@@ -49,7 +49,7 @@ template <typename T, bool C2, bool SPLIT, int PER_SM = 12>
 __global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const bool room, const T* __restrict__ x, int C, int HW, int Cw, long long npix,
                                                                uint64_t* __restrict__ packed) {
   if (room) chain_trigger();
-  chain_wait();
+  x = chain_wait_for(x);
   extern __shared__ __align__(16) uint64_t s_words[];  // [128][CwL]
   const int CwL = SPLIT ? Cw / gridDim.y : Cw, cw0 = SPLIT ? blockIdx.y * CwL : 0;  // this CTA's words of each pixel
   uint16_t* s_q = reinterpret_cast<uint16_t*>(s_words);
@@ -144,7 +144,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) pack_nchw_tile(const bool room, const T* __restrict__ x, int C, int HW, int Cw,
                                                       uint64_t* __restrict__ packed) {
   if (room) chain_trigger();
-  chain_wait();
+  x = chain_wait_for(x);
   __shared__ unsigned char s_sign[64 * 128];
   const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
   const int n = blockIdx.y, p0 = blockIdx.x * 128, cw = blockIdx.z;
@@ -303,7 +303,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) pack_nhwc_c64(const bool room, const T* __restrict__ x, long long total_words,
                                                      uint64_t* __restrict__ packed) {
   if (room) chain_trigger();
-  chain_wait();
+  x = chain_wait_for(x);
   const int lane = threadIdx.x & 31;
   const long long warp_global = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;

@@ -28,3 +28,16 @@ def test_bounded_waits_are_answered_by_the_warp():
     for m in re.finditer(r"\*s_fail != 0", kernel):
         line = kernel[kernel.rfind("\n", 0, m.start()) + 1:kernel.index("\n", m.end())]
         assert "__any_sync(0xFFFFFFFFu, *s_fail != 0)" in line or "*s_fail != 0 && tid == 0" in line, line
+
+
+def test_pointers_to_the_previous_kernel_s_output_come_through_the_wait():
+    """Loads through a const __restrict__ pointer count as invariant and may move above a chained launch's wait.  In the packs, whose
+    input is such a pointer, the wait therefore hands out the pointer that is read."""
+    text = source("pack.cu")
+    kernels = [k for k in re.split(r"(?=template <|__global__)", text) if k.startswith("__global__") and "chain_trigger()" in k]
+    assert len(kernels) == 6
+    for k in kernels:
+        assert "const T* __restrict__ x" in k and "x = chain_wait_for(x);" in k and "chain_wait();" not in k, k[:200]
+        body = k[k.index("{"):]
+        before = body[:body.index("x = chain_wait_for(x);")]
+        assert not re.search(r"\bx\b", before), before
