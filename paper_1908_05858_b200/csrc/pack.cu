@@ -350,6 +350,8 @@ __global__ void pack_weights_kernel(const float* __restrict__ w, int O, int C, i
 
 using namespace dabnn;
 
+namespace {
+
 // NHWC rows of no whole words: one contiguous run per CTA (pack_nhwc_flat) or one thread per word (pack_generic), which reads each
 // lane's row on its own.  The latter stays ahead where a row is short (17 channels, 200704 pixels: 4.27 against 5.44 us) and the pixels
 // many (38 channels, 33504 pixels: 3.64 against 4.98) or few (40 channels, 25 pixels: 2.43 / 2.85; 600 pixels of 39 channels: 3.72 /
@@ -430,6 +432,8 @@ dabnn_status pack_any(const T* x, dabnn_layout in_layout, dabnn_shape s, uint64_
   }
   return launch_status();
 }
+
+}  // namespace
 
 extern "C" dabnn_status dabnn_pack(const float* x, dabnn_layout in_layout, dabnn_shape s, uint64_t* packed,
                                    void* stream) {

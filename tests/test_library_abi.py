@@ -3,6 +3,8 @@ arguments before launching anything."""
 import ctypes
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
 
@@ -32,6 +34,19 @@ def test_every_declared_symbol_is_exported(L):
     for n in names:
         assert hasattr(L, n), n
     assert set(binding.EXPORTS) == set(names)
+
+
+def test_no_bare_names_are_exported(L):
+    """Only the C ABI and names in the library's own namespace can meet those of the program that loads it."""
+    for name in ("_Z4room4dim311dabnn_shape", "_Z14nhwc_flat_paysxi"):
+        assert not hasattr(L, name), name
+    tool = shutil.which("nm")
+    if tool:
+        listed = subprocess.run([tool, "-D", "--defined-only", L._name], capture_output=True, text=True, check=True).stdout
+        names = [line.split()[-1] for line in listed.splitlines()]
+        assert len(names) > 30
+        bare = [n for n in names if not n.startswith("dabnn_") and "5dabnn" not in n and n not in ("_init", "_fini")]
+        assert not bare, bare
 
 
 def test_helpers(L):
