@@ -918,10 +918,17 @@ struct Workspace {
   size_t stem_out, res_a, res_b, bits_a, bits_b, gap, total;
 };
 
+// Up to this many images the 7x7 stem may run as two kernels with the 112x112x64 tensor between them in the workspace; from there on
+// it is always the fused one, and that space holds no more than the STEM module's two tensors.
+constexpr int kTwoKernelStemImages = 3;
+constexpr size_t kStemBytes = (size_t)112 * 112 * 64 * 4, kModuleBytes = (size_t)(112 * 112 * 16 + 56 * 56 * 64) * 4;
+
 Workspace plan(int N) {
   Workspace ws;
   size_t off = 0;
-  ws.stem_out = off; off = align_up(off + (size_t)N * 112 * 112 * 64 * 4, 256);
+  // (the larger of both, so that a workspace for N images also does for fewer)
+  const size_t two_kernels = (N < kTwoKernelStemImages ? N : kTwoKernelStemImages) * kStemBytes, module = N * kModuleBytes;
+  ws.stem_out = off; off = align_up(off + (two_kernels > module ? two_kernels : module), 256);
   ws.res_a = off;    off = align_up(off + (size_t)N * 56 * 56 * 64 * 4, 256);
   ws.res_b = off;    off = align_up(off + (size_t)N * 28 * 28 * 128 * 4, 256);
   ws.bits_a = off;   off = align_up(off + (size_t)N * 56 * 56 * 8, 256);
@@ -1069,7 +1076,7 @@ static dabnn_status forward_impl(const dabnn_bireal18_params* p, const dabnn_ste
     // 150 fused; 4: 167 and 166); below 7 rows per SM two CTAs share a row's channels, so that ranges differ by half a row at
     // most (16 images: 298 us with 64 channels per CTA, 295 with 32; 20: 324 and 325; 128: 1133 and 1169, with two kernels 1298).
     const long long rows = (long long)N * 56, sms_here = sm_count();
-    if (2 * rows >= 3 * sms_here) {
+    if (N > kTwoKernelStemImages || 2 * rows >= 3 * sms_here) {  // (148 SMs: the same bound)
       s = rows >= 7 * sms_here ? launch_stem_pool<8>(p, images, N, cur, bits_in, st) : launch_stem_pool<4>(p, images, N, cur, bits_in, st);
       if (s != DABNN_OK) return s;
     } else {

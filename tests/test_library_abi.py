@@ -63,6 +63,15 @@ def test_helpers(L):
     per1 = L.dabnn_bireal18_workspace_bytes(1)
     assert per1 >= 112 * 112 * 64 * 4 + 56 * 56 * 64 * 4
     assert L.dabnn_bireal18_workspace_bytes(4) <= 4 * per1 + 4096
+    # the stem's 112x112x64 tensor exists up to three images; beyond, its space is the STEM module's 112x112x16 and 56x56x64
+    sizes = [L.dabnn_bireal18_workspace_bytes(N) for N in range(1, 301)]
+    rest = (56 * 56 * 64 + 28 * 28 * 128 + 512) * 4 + 2 * 56 * 56 * 8
+    assert sizes == sorted(sizes)  # a workspace for N images does for fewer
+    for N in (1, 2, 3):
+        assert sizes[N - 1] >= N * (112 * 112 * 64 * 4 + rest)
+    for N in (4, 6, 7, 128, 300):
+        stem = max(3 * 112 * 112 * 64, N * (112 * 112 * 16 + 56 * 56 * 64)) * 4
+        assert stem + N * rest <= sizes[N - 1] <= stem + N * rest + 6 * 256
 
 
 def test_argument_errors_are_reported_before_any_launch(L):
