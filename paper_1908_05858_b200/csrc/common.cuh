@@ -55,8 +55,8 @@ extern thread_local bool g_chain_launch;  // per host thread: set by a forward c
 
 // The calls of the C ABI are chained too (launch_next), but know nothing of what ran before: the caller may have packed the weights
 // a moment ago.  Their kernels touch no global memory before the wait -- they only get themselves onto the SMs, set up tensor
-// memory, barriers and indices while the previous kernel drains.  A kernel lets its successor in early (chain_trigger) only where
-// every SM has room for it then: the CTAs of a successor that come in as SMs empty one by one settle on the first of them (1x1,
+// memory, barriers and indices while the previous kernel drains.  A kernel lets its successor in early (chain_trigger) only behind
+// its main work, and where every SM has room for it then: the CTAs of a successor that come in as SMs empty one by one settle on the first of them (1x1,
 // 512 -> 2048, batch 256: a pack of 392 CTAs, let in by the convolution before it at its start or end, made the pair take 124 or 76 us,
 // 58.5 when it came in at the end of that convolution; 63 with ordinary launches).
 // A kernel that does not take part sees ordinary stream order on both sides.  DABNN_NO_CHAIN in the environment (read once) keeps
