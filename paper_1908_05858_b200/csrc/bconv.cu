@@ -180,8 +180,9 @@ bool tensor_route(const uint64_t* w) {
 }  // namespace
 
 // Fitted (least squares of the relative error; 90 % of the launches within -12 and +12 %) to 3304 launches, those that the tensor-core
-// engine's estimate was fitted to and as many others.  What the two estimates choose together takes 0.5 % longer on the mean
-// than the better engine (0.3 % over 1x1 and 3x3 filters), and 2 % of the launches lose more than 5 %; an estimate from the number
+// engine's estimate was fitted to and as many others, of an earlier form of both kernels and without chained launches.  What the two
+// estimates chose together took 0.5 % longer on the mean than the better engine then, and 2 % of the launches lost more than 5 %.  Of the
+// present kernels, chained, over 320 launches of 1x1 and 3x3 filters: 0.2 %, 5 lose more than 5 %, the worst 11 %.  An estimate from the number
 // of outputs alone, which saw neither the channels beyond O of a tile, nor padding slots, nor how rows leave, lost 4.9 % on the
 // mean, more than 5 % in 10 % of the launches and up to a factor of 3.3.
 // E.g. 3x3 with 256 channels at 14x14: batch 4 6.9 us here, 8.1 there; batch 8 8.6 / 8.1; batch 64 42.0 / 10.9.  64 channels at 56x56,

@@ -1599,7 +1599,8 @@ double tc_plan(TcArgs& g, int epi, int sms) {
   nres = best_n;
   g.nres = (int)nres;
   g.n_groups = (g.n_ntiles + g.nres - 1) / g.nres;
-  // The estimate, fitted (least squares of the relative error; 90 % of the launches within -27 and +18 %) to 1619 launches: 1 to
+  // The estimate, fitted (least squares of the relative error; 90 % of the launches within -27 and +18 %) to 1619 launches of an earlier
+  // form of the kernel, not chained (what it chooses now: see int_pipes_us): 1 to
   // 9216 channels, filters of 1 to 9 rows and columns, strides 1 and 2, images of 1 to 224 pixels a side, O 1 to 4096, every output
   // form, outputs at 4-, 8-, 16- and 32-byte offsets.
   const double live = (double)(nres * g.ntile < o_cols ? nres * g.ntile : o_cols) / 128;

@@ -313,8 +313,8 @@ __global__ void __launch_bounds__(256, 1) stem_pool(const float* __restrict__ im
               w2[2 * h] = pack_f32x2(t4.x, t4.y);
               w2[2 * h + 1] = pack_f32x2(t4.z, t4.w);
             }
-            // (channel pairs outside, pixels inside, the weights as the first factor: which register banks meet decides the rate;
-            // pixels outside: 544 us instead of 528 at batch 128)
+            // (channel pairs outside, pixels inside, the weights as the first factor; pixels outside: 544 us instead of 528 at batch 128,
+            // by the banks of the registers that meet in an instruction, presumably)
 #pragma unroll
             for (int j = 0; j < CPT / 2; j++)
 #pragma unroll

@@ -37,13 +37,14 @@ __device__ __forceinline__ unsigned neg(int32_t v) { return (unsigned)(v < 0); }
 // NCHW, H*W a multiple of 4, 16-byte aligned input.  A CTA covers 128 consecutive pixels of the batch (images follow one
 // another in the pixel count: a tile may span two or more images, so small images leave no ragged tile per image) and all
 // channels.  Each lane owns 4 consecutive pixels of one image (one float4 per channel); the four warps split every word's
-// 64 channels into quarters of 16, so a thread has 16 independent 16-byte loads in flight per word, and the 16-bit
-// quarters are placed side by side in shared memory, which assembles the 64-bit words without any exchange.
+// 64 channels into quarters of 16, so a thread has 16 independent 16-byte loads per word, of which as many are in flight as its
+// registers hold, and the 16-bit quarters are placed side by side in shared memory, which assembles the 64-bit words without any
+// exchange.
 // C2: the words leave in the NC1HWC2 layout instead ([N][C1][H][W][2]: 128-bit vectors of one channel group, pixel after
 // pixel; an odd last word gets a zero partner).
 // SPLIT: gridDim.y CTAs share the words of 128 pixels, for tensors of few pixels and many channels, whose words one CTA packs one after
-// another, a load latency each.  512 channels at 14x14 (HBM floor in brackets): batch 256 25.6 -> 16.4 us (15.7), 64 22.3 -> 5.8 (3.9),
-// 16 22.3 -> 4.3 (1.0).  (PER_SM: twelve CTAs with 40 registers; with 42 the large tensors take 5
+// another, a load latency each.  512 channels at 14x14, packs in a row on inputs in turn (HBM floor in brackets): batch 256 26.3 -> 17.8
+// us (15.7), 64 22.5 -> 6.0 (3.9), 16 10.8 -> 2.7 (1.0; inputs that L2 holds).  (PER_SM: twelve CTAs with 40 registers; with 42 the large tensors take 5
 // us of 68 more.  Split launches that ten per SM hold are 5 to 10 % faster without that limit.)
 template <typename T, bool C2, bool SPLIT, int PER_SM = 12>
 __global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const bool room, const T* __restrict__ x, int C, int HW, int Cw, long long npix,
