@@ -47,6 +47,8 @@ enum { EPI_I32 = 0, EPI_BNPACK = 1, EPI_BIREAL = 2 };
 
 constexpr int TC_THREADS = 416;           // warps 0-3 and (optionally) 8-11: epilogue, 4-7: producers, 12: MMA issue
 constexpr int TC_SMEM_LIMIT = 232448;     // 227 KB opt-in maximum per CTA
+constexpr int TC_SMEM_ALONE = TC_SMEM_LIMIT / 2 + 1024;  // what no two CTAs of an SM (228 KB, 1 KB of each CTA's reserved) can have
+static_assert(2 * (TC_SMEM_ALONE + 1024) > 228 * 1024, "one CTA per SM");
 constexpr int TC_MAX_RES = 4;              // channel tiles resident per CTA (pair) at most
 constexpr int TC_SMEM_HDR = 512;           // barriers, TMEM base, flags
 constexpr int TC_SMEM_MISC = TC_SMEM_HDR + 2 * TC_MAX_RES * 128 * 4;  // ... and this CTA's scale / shift
@@ -1344,6 +1346,10 @@ dabnn_status tc_launch(const TcArgs& g, size_t smem, cudaStream_t st) {
     const int capped = PAIR ? g_tc_max_ctas / 2 : g_tc_max_ctas;
     if (capped < avail) avail = capped > g.n_groups ? capped : g.n_groups;
   }
+  // A CTA takes all of an SM's tensor memory, so a second one there would wait for the first to end.  Instances of 64 registers and
+  // little shared memory would fit twice, and do come to lie on one SM where a launch starts while the kernel before it holds others
+  // (3x3, 64 -> 512, batch 46 at 14x14, int32, with a pack that lets it in at its start 16.3 us, 11.0 like this).
+  if (smem < (size_t)TC_SMEM_ALONE) smem = TC_SMEM_ALONE;
   const long long cap = (long long)avail / g.n_groups * g.n_groups;
   if (cap <= 0) return DABNN_ERR_UNSUPPORTED;
   if (units > cap) units = cap;

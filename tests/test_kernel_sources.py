@@ -52,3 +52,11 @@ def test_packs_let_their_successor_in_behind_their_loads():
         at = body.index("chain_trigger()")
         assert body.count("chain_trigger()") == 1
         assert not re.search(r"\b(x|xn|src|row)\s*(\[|\+)|ld_stream_v4\(|__ldcs\(", body[at:]), body[at:at + 200]
+
+
+def test_a_tensor_core_cta_has_its_sm_alone():
+    """Every launch asks for more shared memory than two CTAs of an SM can have: each takes all of the tensor memory there."""
+    text = source("bconv_tc.cu")
+    assert "static_assert(2 * (TC_SMEM_ALONE + 1024) > 228 * 1024" in text
+    launch = text[text.index("dabnn_status tc_launch(const TcArgs& g"):]
+    assert launch.index("smem = TC_SMEM_ALONE;") < launch.index("<<<")
