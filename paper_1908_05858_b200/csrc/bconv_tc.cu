@@ -140,29 +140,35 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 // The same by a whole warp, whose lanes stay together: every poll's answer is the warp's (1x1, 512 -> 2048, batch 256, sign words with
-// the pack: 51.0 us with an answer per lane, 51.1 like this).  CLUSTER: the arrivals may come from the peer CTA.
-template <bool CLUSTER>
+// the pack: 51.0 us with an answer per lane, 51.1 like this).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* fail, int limit) {
   for (int tries = 0; tries < limit; tries++) {
     uint32_t done;
-    if (CLUSTER)
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t"
-          "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 0x400;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(done)
-          : "r"(bar), "r"(parity)
-          : "memory");
-    else
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t"
-          "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x400;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(done)
-          : "r"(bar), "r"(parity)
-          : "memory");
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x400;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
     if (__all_sync(0xFFFFFFFFu, done != 0)) return true;
     if ((tries & 1023) == 1023 && __any_sync(0xFFFFFFFFu, *fail != 0)) return false;
+  }
+  return false;
+}
+// By one lane, with cluster-scope acquire: the arrivals may come from the peer CTA.
+__device__ __forceinline__ bool mbar_wait_lane_cluster(uint32_t bar, uint32_t parity, volatile int* fail, int limit) {
+  for (int tries = 0; tries < limit; tries++) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 0x400;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((tries & 1023) == 1023 && *fail != 0) return false;
   }
   return false;
 }
@@ -377,7 +383,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   // of its row's 128 channels and stores them as one 16-byte piece instead of four 4-byte ones.  1x1, 512 -> 2048 channels at
   // 14x14, batch 256, with its pack: 79.9 -> 75.1 us.
   constexpr bool ALTERNATE = EPI == EPI_BNPACK && NT == 128;
-  const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;  // (warp: known to be warp-uniform)
+  // (known to be warp-uniform: the issue loop's addresses then are.  Not in the residual form of pairs, which has no use for it and takes
+  // 43.0 us instead of 40.6 with it: 512 channels at 11x11, batch 133)
+  constexpr bool UNIFORM = !(PAIR && EPI == EPI_BIREAL);
+  const int tid = threadIdx.x, warp = UNIFORM ? __shfl_sync(0xFFFFFFFFu, tid >> 5, 0) : tid >> 5, lane = tid & 31;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // 0: the CTA that issues the pair's MMAs
   const int Kb = g.kh * g.kw * (g.C >> 1);               // bytes per weight row
   const int a_bytes = KG ? g.slots * g.gw * 32 : g.slots * (g.C >> 1);  // bytes of one A buffer (one channel group)
@@ -548,7 +557,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
     else __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
-  const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, EARLY && is_producer ? 0u : *tmem_slot, 0);  // (early producers never touch tensor memory)
+  const uint32_t tmem_own = EARLY && is_producer ? 0u : *tmem_slot;  // (early producers never touch tensor memory)
+  const uint32_t tmem_base = UNIFORM ? __shfl_sync(0xFFFFFFFFu, tmem_own, 0) : tmem_own;
   // barriers that both CTAs of a pair signal live in the leader
   const uint32_t bar_tmem_free0 = PAIR ? leader_addr(smem_u32(&bars[B_TMEM_FREE])) : smem_u32(&bars[B_TMEM_FREE]);
   const uint32_t bar_a_full0 = PAIR ? leader_addr(smem_u32(&bars[B_A_FULL])) : smem_u32(&bars[B_A_FULL]);
@@ -578,14 +588,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
   // memory.  A no-op in an ordinary launch.)
 
   if (warp == 12) {
-    // ================= MMA issue: one warp (of the leader CTA), one elected lane per instruction ===================
-    // The warp stays whole, so that addresses and descriptors live in uniform registers: with the loop in one lane every MMA cost
+    // ================= MMA issue: one warp, one elected lane per instruction (in a pair: one lane of the leader) =====
+    // The warp of a single CTA stays whole, so that addresses and descriptors live in uniform registers: with the loop in one lane every MMA cost
     // 120 cycles to issue where an accumulator takes few (1x1, K = 512), against 64 of the tensor pipe; 87 like this.
-    // 3x3, 256 -> 256 at 28x28, batch 256, sign words: 54.8 -> 47.6 us.
+    // 3x3, 256 -> 256 at 28x28, batch 256, sign words: 52.9 -> 45.5 us.
+    // CTA pairs issue from one lane: their MMAs take twice as long, and with the whole warp on it they are slower (512 channels, 3x3:
+    // sign words, batch 8 at 56x56 37.0 -> 38.7 us; int32, batch 35 at 10x10 12.3 -> 12.6; residual form, batch 133 at 11x11 43.0 -> 43.9).
     // The chain below is all there is between two MMAs of this CTA, so it is kept to 32-bit adds: only the start-address
     // field (low 14 bits of a descriptor's low word) changes from one MMA to the next, and shared-memory addresses in
     // 16-byte units never carry out of it.
-    if (rank == 0) {
+    if (rank == 0 && (!PAIR || lane == 0)) {
       const uint32_t idesc = (1u << 7) | (1u << 10)          // A, B: e2m1
                              | ((uint32_t)(NT >> 3) << 17)   // N
                              | (1u << 23)                    // scale factors: ue8m0
@@ -606,7 +618,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         return plane * (uint32_t)g.slots_p + (uint32_t)((ti >> sshift) * g.SP + (tj >> sshift));
       };
       auto mma = [&](uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate) {
-        if (!elect_one()) return;
+        if (!PAIR && !elect_one()) return;
         if (PAIR) {
           asm volatile(
               "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
@@ -625,7 +637,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       };
       // completion of everything issued so far -> one arrival on the barrier at this offset (in both CTAs of a pair)
       auto commit = [&](uint32_t bar) {
-        if (!elect_one()) return;
+        if (!PAIR && !elect_one()) return;
         if (PAIR)
           asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
                        "h"((uint16_t)3)
@@ -633,9 +645,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         else
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
       };
-      // (the warp's answer, poll by poll: a lane's own, at the limit of the polls or when another role has given up, could part the
+      // (a warp's answer, poll by poll: a lane's own, at the limit of the polls or when another role has given up, could part the
       // lanes, and elect_one() takes all of them)
-      auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait_warp<PAIR>(bar, parity, s_fail, g.wait_polls); };
+      auto wait = [&](uint32_t bar, uint32_t parity) {
+        return PAIR ? mbar_wait_lane_cluster(bar, parity, s_fail, g.wait_polls) : mbar_wait_warp(bar, parity, s_fail, g.wait_polls);
+      };
       const bool k3 = g.kh == 3 && g.kw == 3;
       uint32_t off9[9];
 #pragma unroll
@@ -740,13 +754,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
         commit(smem_u32(&bars[B_A_FREE + ab]));  // the tile's rows have been read: the A buffer may be refilled
         if (++ab == (uint32_t)g.abufs) { ab = 0; a_phase ^= 1u; }
       }
-      if (__any_sync(0xFFFFFFFFu, *s_fail != 0)) {  // MMAs of earlier tiles may still read shared memory and write accumulators
+      if (PAIR ? *s_fail != 0 : __any_sync(0xFFFFFFFFu, *s_fail != 0) != 0) {  // MMAs of earlier tiles may still read shared memory and write accumulators
         const uint32_t bar = smem_u32(&bars[B_DRAIN]);
-        if (elect_one()) {
+        if (PAIR || elect_one()) {
           if (PAIR) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
           else asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
         }
-        __syncwarp();
+        if (!PAIR) __syncwarp();
         mbar_drain(smem_u32(&bars[B_DRAIN]), 0);
       }
     }
@@ -1047,7 +1061,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) bconv_tc_kernel(const __grid_co
       const long long m = my_m;
       if constexpr (ALTERNATE) {
         // The next 32 columns and this chunk's thresholds are on their way while a chunk's signs are gathered, and the accumulator
-        // goes back with its last columns in registers.  1x1, 512 -> 2048 at 14x14, batch 256: 45.5 -> 37.4 us (with this warp's
+        // goes back with its last columns in registers.  1x1, 512 -> 2048 at 14x14, batch 256: 44.5 -> 33.1 us, with the issue loop's share (with this warp's
         // loads and thresholds waited for in turn, and a compare and a select per sign, before).
         const uint32_t taddr = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(buf * NT);
         uint32_t va[32], vb[32], words[4];

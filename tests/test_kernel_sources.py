@@ -19,7 +19,10 @@ def test_bounded_waits_are_answered_by_the_warp():
     warp_wait = warp_wait[:warp_wait.index("\n}")]
     assert "if (__all_sync(0xFFFFFFFFu, done != 0)) return true;" in warp_wait and "__any_sync(0xFFFFFFFFu, *fail != 0)" in warp_wait
     kernel = text[text.index("bconv_tc_kernel("):text.index("tc_prepare_weights_kernel")]
-    assert "mbar_wait_warp<PAIR>(" in kernel  # the role that issues the MMAs
+    # the role that issues the MMAs: a whole warp, or one lane of a pair's leader
+    assert "if (rank == 0 && (!PAIR || lane == 0)) {" in kernel
+    assert "return PAIR ? mbar_wait_lane_cluster(bar, parity, s_fail, g.wait_polls) : mbar_wait_warp(bar, parity, s_fail, g.wait_polls);" in kernel
+    kernel = kernel.replace("PAIR ? mbar_wait_lane_cluster(", "").replace("mbar_wait_warp(", "").replace("PAIR ? *s_fail != 0 : ", "")
     calls = [m.start() for m in re.finditer(r"\bmbar_wait\w*\(", kernel)]
     assert len(calls) >= 5
     for at in calls:
