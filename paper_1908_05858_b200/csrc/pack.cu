@@ -47,8 +47,9 @@ __device__ __forceinline__ unsigned neg(int32_t v) { return (unsigned)(v < 0); }
 // us (15.7), 64 22.5 -> 6.0 (3.9), 16 10.8 -> 2.7 (1.0; inputs that L2 holds).  (PER_SM: twelve CTAs with 40 registers; with 42 the large tensors take 5
 // us of 68 more.  Split launches that ten per SM hold are 5 to 10 % faster without that limit.)
 template <typename T, bool C2, bool SPLIT, int PER_SM = 12>
-__global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const bool room, const T* __restrict__ x, int C, int HW, int Cw, long long npix,
+__global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const int room, const T* __restrict__ x, int C, int HW, int Cw, long long npix,
                                                                uint64_t* __restrict__ packed) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   extern __shared__ __align__(16) uint64_t s_words[];  // [128][CwL]
   const int CwL = SPLIT ? Cw / gridDim.y : Cw, cw0 = SPLIT ? blockIdx.y * CwL : 0;  // this CTA's words of each pixel
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const boo
     s_q[((lp + 2) * CwL + cw) * 4 + warp] = (uint16_t)b2;
     s_q[((lp + 3) * CwL + cw) * 4 + warp] = (uint16_t)b3;
   }
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
   __syncthreads();
   const int npx = (int)min((long long)128, npix - pix0);
   if (npx <= 0) return;
@@ -142,8 +143,9 @@ __global__ void __launch_bounds__(kPackThreads, PER_SM) pack_nchw_vec4(const boo
 // 64 x 128 sign flags are gathered with coalesced scalar loads (lanes along pixels) into shared memory; each
 // thread then assembles 32 channel bits of one pixel and stores that half word.
 template <typename T>
-__global__ void __launch_bounds__(256) pack_nchw_tile(const bool room, const T* __restrict__ x, int C, int HW, int Cw,
+__global__ void __launch_bounds__(256) pack_nchw_tile(const int room, const T* __restrict__ x, int C, int HW, int Cw,
                                                       uint64_t* __restrict__ packed) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   __shared__ unsigned char s_sign[64 * 128];
   const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(256) pack_nchw_tile(const bool room, const T* 
       s_sign[c * 128 + p] = (c < cn && p < npix) ? (unsigned char)neg(__ldcs(row + p)) : (unsigned char)0;
     }
   }
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
   __syncthreads();
   const int p = tid & 127, half = tid >> 7;
   if (p < npix) {
@@ -177,7 +179,8 @@ __global__ void __launch_bounds__(256) pack_nchw_tile(const bool room, const T* 
 // each thread gathers 32 channels of one pixel (consecutive lanes: consecutive bytes).  The 128-pixel tiles of the kernel above
 // would leave 79 of 128 lanes idle at 7 x 7.
 template <typename T>
-__global__ void __launch_bounds__(256) pack_nchw_small(const bool room, const T* __restrict__ x, int C, int HW, int Cw, uint64_t* __restrict__ packed) {
+__global__ void __launch_bounds__(256) pack_nchw_small(const int room, const T* __restrict__ x, int C, int HW, int Cw, uint64_t* __restrict__ packed) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   extern __shared__ __align__(16) unsigned char s_flag[];  // [64 * HW]
   using V4 = typename Vec4<T>::type;
@@ -196,7 +199,7 @@ __global__ void __launch_bounds__(256) pack_nchw_small(const bool room, const T*
         reinterpret_cast<uint32_t*>(s_flag)[i0 + u * 256 + tid] = neg(v[u].x) | (neg(v[u].y) << 8) | (neg(v[u].z) << 16) | (neg(v[u].w) << 24);
   }
   if (tid < (count & 3)) s_flag[(count & ~3) + tid] = (unsigned char)neg(src[(count & ~3) + tid]);
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
   __syncthreads();
   for (int i = tid; i < 2 * HW; i += 256) {
     const int half = i >= HW ? 1 : 0, p = i - half * HW;
@@ -218,8 +221,9 @@ __global__ void __launch_bounds__(256) pack_nchw_small(const bool room, const T*
 // half k of pixel p is then the bit field of 32 (or what is left of C) bits that starts at bit p * C + 32 * k: one funnel
 // shift, stored by consecutive threads to consecutive addresses.
 template <typename T>
-__global__ void __launch_bounds__(256) pack_nhwc_flat(const bool room, const T* __restrict__ x, int C, int P, int halves, long long npix,
+__global__ void __launch_bounds__(256) pack_nhwc_flat(const int room, const T* __restrict__ x, int C, int P, int halves, long long npix,
                                                       uint32_t* __restrict__ packed) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   extern __shared__ __align__(16) uint32_t s_bits[];  // [P * C / 32 + 1]
   using V4 = typename Vec4<T>::type;
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(256) pack_nhwc_flat(const bool room, const T* 
       if ((lane & 7) == 0 && i < count4) s_bits[i >> 3] = word;
     }
   }
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
   __syncthreads();
   uint32_t* dst = packed + p0 * halves;
   for (int i = tid; i < np * halves; i += 256) {
@@ -269,8 +273,9 @@ __global__ void __launch_bounds__(256) pack_nhwc_flat(const bool room, const T* 
 // Any layout, any shape: one thread per output word (c2: the word goes to its place in the NC1HWC2 layout, and the
 // thread of an odd last word also writes the zero partner).
 template <typename T>
-__global__ void pack_generic(const bool room, const T* __restrict__ x, int nhwc, int C, int HW, int Cw, long long total_words,
+__global__ void pack_generic(const int room, const T* __restrict__ x, int nhwc, int C, int HW, int Cw, long long total_words,
                              uint64_t* __restrict__ packed, int c2) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total_words) return;
@@ -286,7 +291,7 @@ __global__ void pack_generic(const bool room, const T* __restrict__ x, int nhwc,
     const T* src = x + ((size_t)n * C + c0) * HW + hw;
     for (int c = 0; c < cn; c++) w |= (uint64_t)neg(src[(size_t)c * HW]) << c;
   }
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
   if (c2) {
     const long long n = pix / HW, hw = pix % HW;
     const int C1 = (Cw + 1) / 2;
@@ -301,8 +306,9 @@ __global__ void pack_generic(const bool room, const T* __restrict__ x, int nhwc,
 // NHWC with C a multiple of 64 and 16-byte aligned input: 16 lanes share one word; each lane tests 4
 // channels (one float4), places its nibble, and an OR-reduction over 8-lane groups builds each half.
 template <typename T>
-__global__ void __launch_bounds__(256) pack_nhwc_c64(const bool room, const T* __restrict__ x, long long total_words,
+__global__ void __launch_bounds__(256) pack_nhwc_c64(const int room, const T* __restrict__ x, long long total_words,
                                                      uint64_t* __restrict__ packed) {
+  if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   const int lane = threadIdx.x & 31;
   const long long warp_global = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -327,7 +333,7 @@ __global__ void __launch_bounds__(256) pack_nhwc_c64(const bool room, const T* _
       if ((lane & 15) == 0 && word < total_words) packed[word] = (uint64_t)half | ((uint64_t)other << 32);
     }
   }
-  if (room) chain_trigger();
+  if (room == 1) chain_trigger();
 }
 
 __global__ void pack_weights_kernel(const float* __restrict__ w, int O, int C, int taps, int Cw,
@@ -364,14 +370,17 @@ bool nhwc_flat_pays(long long npix, int C) {
   return (npix < 32 ? npix : 32) * C <= 18000 || npix >= 64 * 32;
 }
 
-// At most four CTAs per SM, half of what it holds, of a pack of a few microseconds: the next kernel of the stream finds room on every
-// SM and may come in behind the loads.  (Of 103 MB in 392 CTAs, packs one after the other: 28 us each, 39 when they let one another
-// in.)  Behind the loads and not at the start: CTAs that come in while most of the pack's are still there settle unevenly.  With its
-// pack, 3x3, let in at the start, behind the loads, at the end: 256 channels at 14x14, batch 8 (integer pipes) 13.1, 10.1 and 10.3 us, at
-// 7x7, batch 40 12.9, 11.3 and 11.6; 64 -> 512 channels at 14x14, batch 46 16.3, 11.3 and 11.5 (tensor engine), 256 channels at 14x14,
-// batch 64 11.5, 12.0 and 12.3.  Packs of 73 x 434 x 7 x 7 one after the other 5.0, 3.7 and 3.9 each.
-bool room(dim3 grid, dabnn_shape s) {
-  return (long long)grid.x * grid.y * grid.z <= 4LL * sm_count() && (long long)s.N * s.C * s.H * s.W <= 4 << 20;
+// When a pack lets the next kernel of the stream in: 0 at its end, 1 behind its loads, 2 at its start.
+// Behind the loads: at most four CTAs per SM, half of what it holds, of a pack of a few microseconds, so that the next kernel finds room on
+// every SM (of 103 MB in 392 CTAs, packs one after the other: 28 us each, 39 when they let one another in).  At the start only where
+// the pack's CTAs are on three SMs in ten at most: CTAs that come in while there are more of them settle unevenly.  With its pack,
+// 3x3, let in at the start, behind the loads, at the end: 256 channels at 14x14, batch 8 (52 CTAs; integer pipes) 13.1, 10.1 and 10.3 us,
+// at 7x7, batch 40 (160) 12.9, 11.3 and 11.6; 128 channels at 14x14, batch 2 (8; tensor engine) 7.4 and 8.2 at the start and behind
+// the loads, 64 -> 256 at 32x32, batch 3 (24) 6.9 and 7.7.  Packs of 73 x 434 x 7 x 7 (511) one after the other 5.0, 3.7 and 3.9 each.
+int room(dim3 grid, dabnn_shape s) {
+  const long long ctas = (long long)grid.x * grid.y * grid.z, sms = sm_count();
+  if ((long long)s.N * s.C * s.H * s.W > 4 << 20 || ctas > 4 * sms) return 0;
+  return 10 * ctas <= 3 * sms ? 2 : 1;
 }
 
 template <typename T>

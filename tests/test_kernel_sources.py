@@ -48,13 +48,14 @@ def test_pointers_to_the_previous_kernel_s_output_come_through_the_wait():
 
 def test_packs_let_their_successor_in_behind_their_loads():
     """CTAs of the next kernel that come in while a pack's are still loading settle unevenly on the SMs (a third more time for a small
-    convolution and its pack): in every pack the trigger stands behind the last read of the input."""
+    convolution and its pack): in every pack the trigger stands behind the last read of the input, but for packs of few CTAs."""
     text = source("pack.cu")
     for k in [k for k in re.split(r"(?=template <|__global__)", text) if k.startswith("__global__") and "chain_trigger()" in k]:
         body = k[k.index("{"):]
-        at = body.index("chain_trigger()")
-        assert body.count("chain_trigger()") == 1
+        assert body.count("chain_trigger()") == 2 and "if (room == 2) chain_trigger();\n  x = chain_wait_for(x);" in body
+        at = body.index("if (room == 1) chain_trigger()")
         assert not re.search(r"\b(x|xn|src|row)\s*(\[|\+)|ld_stream_v4\(|__ldcs\(", body[at:]), body[at:at + 200]
+    assert "return 10 * ctas <= 3 * sms ? 2 : 1;" in text
 
 
 def test_a_tensor_core_cta_has_its_sm_alone():
