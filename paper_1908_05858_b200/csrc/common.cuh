@@ -72,8 +72,10 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // intrinsic is a volatile asm).
 template <typename T>
 __device__ __forceinline__ const T* chain_wait_for(const T* p) {
-  asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
-  return p;
+  size_t g = __cvta_generic_to_global(p);  // (so that the result is known to point to global memory: int32 pack of 119 x 56 x 56 x 70, NHWC,
+                                           // 27.9 us, 30.4 with generic loads)
+  asm volatile("griddepcontrol.wait;" : "+l"(g)::"memory");
+  return static_cast<const T*>(__cvta_global_to_generic(g));
 }
 // ... and for further pointers, behind a wait.
 template <typename T>
