@@ -308,6 +308,7 @@ __global__ void pack_generic(const int room, const T* __restrict__ x, int nhwc, 
 template <typename T>
 __global__ void __launch_bounds__(256) pack_nhwc_c64(const int room, const T* __restrict__ x, long long total_words,
                                                      uint64_t* __restrict__ packed) {
+  // (nothing is left to do behind the loop's last loads: a trigger there gains nothing and costs the loop, 64 x 28 x 28 x 256 11.1 against 10.7 us)
   if (room == 2) chain_trigger();
   x = chain_wait_for(x);
   const int lane = threadIdx.x & 31;
@@ -333,7 +334,6 @@ __global__ void __launch_bounds__(256) pack_nhwc_c64(const int room, const T* __
       if ((lane & 15) == 0 && word < total_words) packed[word] = (uint64_t)half | ((uint64_t)other << 32);
     }
   }
-  if (room == 1) chain_trigger();
 }
 
 __global__ void pack_weights_kernel(const float* __restrict__ w, int O, int C, int taps, int Cw,

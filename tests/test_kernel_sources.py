@@ -52,7 +52,11 @@ def test_packs_let_their_successor_in_behind_their_loads():
     text = source("pack.cu")
     for k in [k for k in re.split(r"(?=template <|__global__)", text) if k.startswith("__global__") and "chain_trigger()" in k]:
         body = k[k.index("{"):]
-        assert body.count("chain_trigger()") == 2 and "if (room == 2) chain_trigger();\n  x = chain_wait_for(x);" in body
+        assert "if (room == 2) chain_trigger();\n  x = chain_wait_for(x);" in body
+        if "pack_nhwc_c64" in k:  # (lets the next kernel in at its end)
+            assert body.count("chain_trigger()") == 1
+            continue
+        assert body.count("chain_trigger()") == 2
         at = body.index("if (room == 1) chain_trigger()")
         assert not re.search(r"\b(x|xn|src|row)\s*(\[|\+)|ld_stream_v4\(|__ldcs\(", body[at:]), body[at:at + 200]
     assert "return 10 * ctas <= 3 * sms ? 2 : 1;" in text
